@@ -223,11 +223,15 @@ struct PintGeom {
   int cta_sum;   // 1: the teams of a CTA add their partial rows (nblk == 1)
   int acc_rows;  // partial rows per block in acc_part (R, or CTAs when cta_sum)
   int stage;     // 1: tau K staged in shared memory once per launch
+  int chunk;     // 1: a geometry of k_pint_chunk (pint_chunk.cu): teams of P >= 8 lanes, a CTA per
+                 // (block, split of the frequencies)
 };
 // m_req / teams_req: rows per thread and teams per CTA requested by the caller (0 = choose);
 // fact: the loops will use stored factors (a smaller shared-memory footprint)
 PintGeom pint_geometry(int nf, int nblk, int blen, int target_teams, int elem_bytes, int m_req = 0,
                        int teams_req = 0, bool fact = false);
+// The geometry of k_pint_chunk, the binary32 loop without stored factors or the FP64 lane.
+PintGeom pint_chunk_geometry(int nf, int nblk, int blen);
 void set_acc_rows(PintGeom &g);  // recompute cta_sum / acc_rows after changing R
 
 template <typename T>
@@ -285,6 +289,7 @@ size_t pint_k0_factor_elems(const PintGeom &g);
 size_t pint_factor_elems(const PintGeom &g);
 template <typename T>
 void launch_pint(Ctx &c, const PintGeom &g, const PintArgs<T> &a);
+void launch_pint_chunk(Ctx &c, const PintGeom &g, const PintArgs<float> &a);
 void launch_recip_f32(cudaStream_t s, const float *x, float *r, int64_t n);
 struct InitTail;  // pd_krylov.cuh: the start of Algorithm 2 run by a reduction's last CTA
 struct ProjTail;  // pd_krylov.cuh: eq. 13 and the step decision run by the z reduction's last CTA

@@ -1000,7 +1000,7 @@ void set_acc_rows(PintGeom &g) {
 
 PintGeom pint_geometry(int nf, int nblk, int blen, int target_teams, int elem_bytes, int m_req, int teams_req,
                        bool fact) {
-  PintGeom g;
+  PintGeom g{};
   g.nf = nf;
   g.nblk = nblk;
   g.blen = blen;
@@ -1059,6 +1059,9 @@ static void launch_pint_m(Ctx &c, const PintGeom &g, const PintArgs<T> &a) {
 
 template <typename T>
 void launch_pint(Ctx &c, const PintGeom &g, const PintArgs<T> &a) {
+  if constexpr (sizeof(T) == 4) {
+    if (g.chunk) return launch_pint_chunk(c, g, a);
+  }
   if (g.M == 4) {
     launch_pint_m<T, 4>(c, g, a);
   } else if (g.M == 16) {

@@ -230,7 +230,8 @@ struct pd_plan {
   void *fac = nullptr;
   double *mscal = nullptr;  // per-problem Algorithm-2 scalar and flag blocks
   int *mflags = nullptr;
-  pd::PintGeom geom{};
+  pd::PintGeom geom{};   // k_pint's teams
+  pd::PintGeom cgeom{};  // k_pint_chunk's teams (chunk = 0: not used by this plan)
   int blas_grid = 1, k5_grid = 1;
   int k5_grid_members = 1;  // capacitance CTAs per problem of a batched plan
   int blas_cluster = 0;  // CTAs of the cluster variant of the one-CTA Krylov kernels (0 = off)
@@ -556,6 +557,11 @@ void fill_geometry(pd_plan *p, const pd_desc *d) {
   const int target = sms * ctas_per_sm * g0.teams_per_cta;
   p->geom =
       pd::pint_geometry(p->nf, p->nblk, p->blen, target, esz, d->tune_pint_rows, d->tune_pint_teams, want_fac);
+  // binary32 loops that eliminate as they solve keep their chunks in registers (pint_chunk.cu),
+  // unless the caller asked for a launch geometry of k_pint
+  p->cgeom = pd::PintGeom{};
+  if (d->precision == PD_MIXED && !want_fac && !d->tune_pint_rows && !d->tune_pint_teams)
+    p->cgeom = pd::pint_chunk_geometry(p->nf, p->nblk, p->blen);
   // Krylov vector kernels: vectors up to 8192 entries run in one 512-thread CTA or (see
   // below) a cluster; beyond, cooperative 64-thread CTAs, at most one per SM (co-resident)
   p->blas_grid =
@@ -709,7 +715,7 @@ size_t layout(pd_plan *p, unsigned char *base) {
   p->b0 = A.take<double>(nbar);
   p->x0 = A.take<double>(nbar);
   p->y = A.take<double>((size_t)(mx + 1) * nmem);
-  p->acc_part = A.take<double>((size_t)p->geom.nblk * p->geom.R * p->geom.blen);
+  p->acc_part = A.take<double>((size_t)p->geom.nblk * std::max(p->geom.R, p->cgeom.R) * p->geom.blen);
   if (mixed) {
     p->acc0 = A.take<double>(nbar);
     p->h0 = A.take<double>(nbar);
@@ -1015,6 +1021,9 @@ pd_status sync_read(pd_plan *p, bool with_tail = false) {
 
 // The final loop by linearity applies to single problems of the full method whose zero
 // frequency runs in binary32 like the others (the FP64 lane keeps the final loop's solves).
+// Geometry of the loops of an Algorithm-1 solve: the FP64 zero-frequency lane is k_pint's.
+const pd::PintGeom &loop_geom(const pd_plan *p) { return p->cgeom.chunk && !p->lane ? p->cgeom : p->geom; }
+
 bool use_comb(const pd_plan *p) { return p->comb && !(p->precision == PD_MIXED && p->lane); }
 
 template <typename T>
@@ -1247,18 +1256,18 @@ pd_status emit_pre(pd_plan *p, int kind, const double *G, double *U, int use_han
     a.Y = L;
     a.ldy = p->lds;
   }
-  pd::launch_pint<T>(c, p->geom, a);
+  pd::launch_pint<T>(c, loop_geom(p), a);
   pd::KrylovBufs kb = kbufs<T>(p);
   double *acc0 = lane_acc0<T>(p);
   if (kb.members) {
-    pd::launch_acc_reduce(c, p->geom, p->acc_part, p->b, nullptr, nullptr, acc0);
+    pd::launch_acc_reduce(c, loop_geom(p), p->acc_part, p->b, nullptr, nullptr, acc0);
     pd::launch_member_init(c, kb, p->b, use_handle, hk);
   } else if (p->krylov_tails) {  // beta and v_1 in the b reduction's last CTA
     const pd::InitTail t{1, p->flags + pd::F_ACCCNT, kb.n, kb.maxit + 2, (kb.maxit + 1) * kb.maxit, use_handle,
                          kb.part, kb.V, kb.scal, kb.T, kb.Vf, kb.flags, hk};
-    pd::launch_acc_reduce(c, p->geom, p->acc_part, p->b, nullptr, &t, acc0);
+    pd::launch_acc_reduce(c, loop_geom(p), p->acc_part, p->b, nullptr, &t, acc0);
   } else {
-    pd::launch_acc_reduce(c, p->geom, p->acc_part, p->b, nullptr, nullptr, acc0);
+    pd::launch_acc_reduce(c, loop_geom(p), p->acc_part, p->b, nullptr, nullptr, acc0);
     pd::launch_vec_norm_init(c, kb, p->b, use_handle, hk);
   }
   // x_m = b: the inner matrix of eq. (17) taken as I (two loops in all)
@@ -1349,7 +1358,7 @@ pd_status emit_iter(pd_plan *p, int kind, int use_handle, cudaGraphConditionalHa
     a.ldy = p->lds;
     a.skip_flag = noh;
     a.h0 = lane_h0<T>(p);
-    pd::launch_pint<T>(c, p->geom, a);
+    pd::launch_pint<T>(c, loop_geom(p), a);
   }
   if (p->persist) {
     pd::launch_step_tail<T>(c, step_args<T>(p, kind, use_handle, hk), p->persist_grid, p->persist_E);
@@ -1407,7 +1416,7 @@ pd_status emit_post(pd_plan *p, int kind, double *U, int use_handle, cudaGraphCo
                              p->x);
     a.skip_flag2 = p->flags + pd::F_COMB;
   }
-  pd::launch_pint<T>(c, p->geom, a);
+  pd::launch_pint<T>(c, loop_geom(p), a);
   if (kind == 0) {
     CK(cudaMemcpyAsync(p->b0, p->b, sizeof(double) * p->nbar, cudaMemcpyDeviceToDevice, c.stream));
     CK(cudaMemcpyAsync(p->x0, p->x, sizeof(double) * p->nbar, cudaMemcpyDeviceToDevice, c.stream));
@@ -2056,9 +2065,9 @@ pd_status paradiag_shifted_solve(pd_plan *p, const void *R, void *Y, double *b) 
       a.omega = p->wg;
       a.acc_part = p->acc_part;
     }
-    pd::launch_pint<float>(p->ctx, p->geom, a);
+    pd::launch_pint<float>(p->ctx, loop_geom(p), a);
   }
-  if (b) pd::launch_acc_reduce(p->ctx, p->geom, p->acc_part, b, nullptr);
+  if (b) pd::launch_acc_reduce(p->ctx, loop_geom(p), p->acc_part, b, nullptr);
   CK(cudaStreamSynchronize(p->ctx.stream));
   return ctx_status(p);
 }
