@@ -211,6 +211,19 @@ void launch_dst_y_residual(Ctx &c, const double *G, const double *U, T *Y, int64
                            int64_t nx, const double *rxl, const double *rdd, const double *rxu, const double *ryl,
                            const double *ryu, const int *mex, const cpx<T> *tw);
 
+// ---- the operator's device arrays (operator.cu) ---------------------------------------
+struct OperatorArgs {
+  int64_t nbar, nrx, ny, nx, nym;
+  double tau;
+  const double *xlo, *xdiag, *xup;              // T_x of every problem (nrx)
+  const double *ylo, *ydiag, *yup, *mu;         // 2D: T_y and the eigenvalue of each row's mode (ny); 1D: null
+  double *klo, *kdiag, *kup;                    // K in the solve basis (nbar)
+  double *tlo_d, *tdiag_d, *tup_d;              // tau K
+  float *tlo_f, *tdiag_f, *tup_f;               // the same in binary32, or null
+  double *rxl, *rxd, *rxu, *ryl, *ryd, *ryu, *rdd;  // residual coefficients
+};
+void launch_operator(Ctx &c, const OperatorArgs &o);
+
 // ---- shifted tridiagonal solves (pint.cu) ------------------------------------------
 struct PintGeom {
   int nf;        // frequencies k = 0..nf-1 (half spectrum)

@@ -257,7 +257,11 @@ struct pd_plan {
   double *klo = nullptr, *kdiag = nullptr, *kup = nullptr;
   double *tlo_d = nullptr, *tdiag_d = nullptr, *tup_d = nullptr;
   float *tlo_f = nullptr, *tdiag_f = nullptr, *tup_f = nullptr;
-  double *xlo = nullptr, *xdiag = nullptr, *xup = nullptr, *ylo = nullptr, *ydiag = nullptr, *yup = nullptr;
+  // compact source of the operator: T_x (lo, diag, up; nrx each), 2D: T_y (lo, diag, up) and the
+  // modes' eigenvalues (ny each); hop and hmsc, hbnx are the host sides of its uploads
+  double *opsrc = nullptr;
+  std::vector<double> hop, hmsc;
+  std::vector<int> hbnx;
   // residual coefficients: (tau lo_x, 1 + tau diag_x, tau up_x) and (tau lo_y, tau diag_y, tau up_y)
   double *rxl = nullptr, *rxd = nullptr, *rxu = nullptr, *ryl = nullptr, *ryd = nullptr, *ryu = nullptr;
   double *rdd = nullptr;  // 2D: rxd + ryd at every point of the grid (n_bar), one FP64 add less per point
@@ -306,10 +310,10 @@ struct pd_plan {
 
 namespace {
 
-// Host copies of the operator in the solve basis.
+// Host copy of the operator: T_x of every problem, and in 2D T_y and mu, the eigenvalue of T_y
+// that the diagonal of each block (one mode of T_y) carries.
 struct HostOp {
-  std::vector<double> lo, diag, up;  // K~ (length nbar), block-decoupled
-  std::vector<double> xlo, xdiag, xup, ylo, ydiag, yup;
+  std::vector<double> xlo, xdiag, xup, ylo, ydiag, yup, mu;
 };
 
 // The shifted solves eliminate without pivoting (partitioned Thomas + PCR).  Every
@@ -666,16 +670,11 @@ size_t layout(pd_plan *p, unsigned char *base) {
     p->tdiag_f = A.take<float>(nbar);
     p->tup_f = A.take<float>(nbar);
   }
-  p->xlo = A.take<double>(p->nrx);
-  p->xdiag = A.take<double>(p->nrx);
-  p->xup = A.take<double>(p->nrx);
+  p->opsrc = A.take<double>(3 * p->nrx + (p->dim == 2 ? 4 * p->ny : 0));
   p->rxl = A.take<double>(p->nrx);
   p->rxd = A.take<double>(p->nrx);
   p->rxu = A.take<double>(p->nrx);
   if (p->dim == 2) {
-    p->ylo = A.take<double>(p->ny);
-    p->ydiag = A.take<double>(p->ny);
-    p->yup = A.take<double>(p->ny);
     p->ryl = A.take<double>(p->ny);
     p->ryd = A.take<double>(p->ny);
     p->rdd = A.take<double>(p->nbar);
@@ -770,9 +769,7 @@ HostOp build_batched_operator_2d(const pd_desc *d) {
   h.ylo.assign(ny * B, 0.0);
   h.ydiag.assign(ny * B, 0.0);
   h.yup.assign(ny * B, 0.0);
-  h.lo.resize(nx * ny * B);
-  h.diag.resize(nx * ny * B);
-  h.up.resize(nx * ny * B);
+  h.mu.assign(ny * B, 0.0);
   for (int64_t b = 0; b < B; ++b) {
     const double tb = d->batch_tau ? d->batch_tau[b] : d->tau;
     for (int64_t i = 0; i < nx; ++i) {
@@ -787,13 +784,7 @@ HostOp build_batched_operator_2d(const pd_desc *d) {
       h.ylo[r] = l > 0 ? tb * d->k_lo_y[r] : 0.0;
       h.ydiag[r] = tb * d->k_diag_y[r];
       h.yup[r] = l + 1 < ny ? tb * d->k_up_y[r] : 0.0;
-      const double mu = tb * (dd + 2.0 * c * std::cos(M_PI * (double)(l + 1) / (double)(ny + 1)));
-      for (int64_t ix = 0; ix < nx; ++ix) {
-        const int64_t j = r * nx + ix;
-        h.lo[j] = h.xlo[b * nx + ix];
-        h.diag[j] = h.xdiag[b * nx + ix] + mu;
-        h.up[j] = h.xup[b * nx + ix];
-      }
+      h.mu[r] = tb * (dd + 2.0 * c * std::cos(M_PI * (double)(l + 1) / (double)(ny + 1)));
     }
   }
   return h;
@@ -818,9 +809,6 @@ HostOp build_batched_operator(const pd_desc *d) {
       h.xup[j] = i + 1 < nb ? tb * d->k_up[j] : 0.0;
     }
   }
-  h.lo = h.xlo;
-  h.diag = h.xdiag;
-  h.up = h.xup;
   return h;
 }
 
@@ -835,9 +823,6 @@ void scale_by_mass(HostOp &h, const double *m) {
     if (j > 0) h.xlo[j] *= s[j] * s[j - 1];
     if (j + 1 < n) h.xup[j] *= s[j] * s[j + 1];
   }
-  h.lo = h.xlo;
-  h.diag = h.xdiag;
-  h.up = h.xup;
 }
 
 HostOp build_operator_plain(const pd_desc *d);
@@ -857,10 +842,6 @@ HostOp build_operator_plain(const pd_desc *d) {
   h.xup.assign(d->k_up, d->k_up + nx);
   h.xlo[0] = 0.0;
   h.xup[nx - 1] = 0.0;
-  h.lo.resize(nx * ny);
-  h.diag.resize(nx * ny);
-  h.up.resize(nx * ny);
-  std::vector<double> mu(ny, 0.0);
   if (d->dim == 2) {
     h.ylo.assign(d->k_lo_y, d->k_lo_y + ny);
     h.ydiag.assign(d->k_diag_y, d->k_diag_y + ny);
@@ -869,15 +850,9 @@ HostOp build_operator_plain(const pd_desc *d) {
     h.yup[ny - 1] = 0.0;
     const double dd = d->k_diag_y[0];
     const double c = ny > 1 ? d->k_up_y[0] : 0.0;
-    for (int64_t l = 0; l < ny; ++l) mu[l] = dd + 2.0 * c * std::cos(M_PI * (double)(l + 1) / (double)(ny + 1));
+    h.mu.resize(ny);
+    for (int64_t l = 0; l < ny; ++l) h.mu[l] = dd + 2.0 * c * std::cos(M_PI * (double)(l + 1) / (double)(ny + 1));
   }
-  for (int64_t l = 0; l < ny; ++l)
-    for (int64_t ix = 0; ix < nx; ++ix) {
-      const int64_t j = l * nx + ix;
-      h.lo[j] = h.xlo[ix];
-      h.diag[j] = h.xdiag[ix] + mu[l];
-      h.up[j] = h.xup[ix];
-    }
   return h;
 }
 
@@ -886,6 +861,8 @@ HostOp build_operator_plain(const pd_desc *d) {
     cudaError_t e_ = (call);                                                                       \
     if (e_ != cudaSuccess) return fail(PD_ERR_CUDA, "%s failed: %s", #call, cudaGetErrorString(e_)); \
   } while (0)
+
+pd_status ctx_status(pd_plan *p);
 
 template <typename X>
 pd_status upload(X *dst, const X *src, size_t n, cudaStream_t s) {
@@ -907,99 +884,112 @@ pd_status upload(X *dst, const X *src, size_t n, cudaStream_t s) {
 // A_0 x = 1 and A_0 x = (-1)^i (exact for M-matrices such as the heat and upwind operators,
 // whose inverses are nonnegative), the largest |x_i| over the blocks, divided by l.
 constexpr double kLaneWeight = 4.0;
-double zero_frequency_weight(const pd_plan *p, const std::vector<double> &tlo, const std::vector<double> &tdiag,
-                             const std::vector<double> &tup) {
+// W blocks side by side: their division chains overlap, and one elimination serves both
+// right-hand sides (a 127 x 127 grid: 0.3 ms block by block, side by side a few hundredths).
+template <int W>
+double thomas_worst(const pd_plan *p, const HostOp &h, int64_t b0, std::vector<double> &work) {
   const double s0 = 1.0 - p->aroot;  // 1 - pi_0
-  const int64_t nb = p->nblk, bl = p->blen;
-  std::vector<double> cp(bl), dp(bl);
-  double worst = 0.0;
-  for (int64_t b = 0; b < nb; ++b) {
-    const int64_t o = b * bl;
-    for (int sign = 0; sign < 2; ++sign) {
-      for (int64_t i = 0; i < bl; ++i) {
-        const double lo = i > 0 ? tlo[o + i] : 0.0, up = i + 1 < bl ? tup[o + i] : 0.0;
-        const double r = (sign && (i & 1)) ? -1.0 : 1.0;
-        const double m = s0 + tdiag[o + i] - (i > 0 ? lo * cp[i - 1] : 0.0);
-        cp[i] = up / m;
-        dp[i] = (r - (i > 0 ? lo * dp[i - 1] : 0.0)) / m;
-      }
-      double x = dp[bl - 1];
-      worst = std::max(worst, std::fabs(x));
-      for (int64_t i = bl - 2; i >= 0; --i) {
-        x = dp[i] - cp[i] * x;
-        worst = std::max(worst, std::fabs(x));
-      }
+  const int64_t bl = p->blen;
+  double *cp = work.data(), *d0 = cp + bl * W, *d1 = d0 + bl * W;
+  int64_t o[W];  // the blocks' x-coefficients and eigenvalues
+  double mu[W];
+  for (int w = 0; w < W; ++w) {
+    o[w] = p->dim == 2 ? (b0 + w) / p->nym * bl : (b0 + w) * bl;
+    mu[w] = p->dim == 2 ? h.mu[b0 + w] : 0.0;
+  }
+  for (int64_t i = 0; i < bl; ++i) {
+    const double r1 = (i & 1) ? -1.0 : 1.0;
+    for (int w = 0; w < W; ++w) {
+      const double lo = i > 0 ? p->tau * h.xlo[o[w] + i] : 0.0, up = i + 1 < bl ? p->tau * h.xup[o[w] + i] : 0.0;
+      const double c = i > 0 ? cp[(i - 1) * W + w] : 0.0;
+      const double a0 = i > 0 ? d0[(i - 1) * W + w] : 0.0, a1 = i > 0 ? d1[(i - 1) * W + w] : 0.0;
+      const double rm = 1.0 / (s0 + p->tau * (h.xdiag[o[w] + i] + mu[w]) - lo * c);
+      cp[i * W + w] = up * rm;
+      d0[i * W + w] = (1.0 - lo * a0) * rm;
+      d1[i * W + w] = (r1 - lo * a1) * rm;
     }
   }
+  double worst[W], x0[W], x1[W];
+  for (int w = 0; w < W; ++w) worst[w] = x0[w] = x1[w] = 0.0;
+  for (int64_t i = bl - 1; i >= 0; --i)
+    for (int w = 0; w < W; ++w) {
+      x0[w] = d0[i * W + w] - cp[i * W + w] * x0[w];
+      x1[w] = d1[i * W + w] - cp[i * W + w] * x1[w];
+      worst[w] = std::max(std::max(worst[w], std::fabs(x0[w])), std::fabs(x1[w]));
+    }
+  return *std::max_element(worst, worst + W);
+}
+
+double zero_frequency_weight(const pd_plan *p, const HostOp &h) {
+  constexpr int W = 8;
+  std::vector<double> work((size_t)3 * p->blen * (p->nblk >= W ? W : 1));
+  double worst = 0.0;
+  int64_t b = 0;
+  for (; b + W <= p->nblk; b += W) worst = std::max(worst, thomas_worst<W>(p, h, b, work));
+  for (; b < p->nblk; ++b) worst = std::max(worst, thomas_worst<1>(p, h, b, work));
   return std::isfinite(worst) ? worst / (double)p->nt : 1e300;
 }
 
 pd_status upload_operator(pd_plan *p, const pd_desc *desc) {
   pd_status st = PD_OK;
-  HostOp h = build_operator(desc);
-  const int64_t nbar = p->nbar;
-  std::vector<double> tlo(nbar), tdiag(nbar), tup(nbar);
-  std::vector<float> flo(nbar), fdiag(nbar), fup(nbar);
-  for (int64_t j = 0; j < nbar; ++j) {
-    tlo[j] = p->tau * h.lo[j];
-    tdiag[j] = p->tau * h.diag[j];
-    tup[j] = p->tau * h.up[j];
-    flo[j] = (float)tlo[j];
-    fdiag[j] = (float)tdiag[j];
-    fup[j] = (float)tup[j];
-  }
-  std::vector<double> rxl(p->nrx), rxd(p->nrx), rxu(p->nrx), ryl(p->ny), ryd(p->ny), ryu(p->ny);
-  for (int64_t i = 0; i < p->nrx; ++i) {
-    rxl[i] = p->tau * h.xlo[i];
-    rxd[i] = 1.0 + p->tau * h.xdiag[i];
-    rxu[i] = p->tau * h.xup[i];
-  }
-  if (p->dim == 2)
-    for (int64_t i = 0; i < p->ny; ++i) {
-      ryl[i] = p->tau * h.ylo[i];
-      ryd[i] = p->tau * h.ydiag[i];
-      ryu[i] = p->tau * h.yup[i];
-    }
+  const HostOp h = build_operator(desc);
   if (p->precision == PD_MIXED) {
-    p->nu0 = zero_frequency_weight(p, tlo, tdiag, tup);
+    p->nu0 = zero_frequency_weight(p, h);
     p->lane = desc->tune_zero_lane > 0 || (desc->tune_zero_lane == 0 && p->nu0 > kLaneWeight);
   }
   cudaStream_t s = p->ctx.stream;
-  if ((st = upload(p->klo, h.lo.data(), nbar, s)) || (st = upload(p->kdiag, h.diag.data(), nbar, s)) ||
-      (st = upload(p->kup, h.up.data(), nbar, s)) || (st = upload(p->tlo_d, tlo.data(), nbar, s)) ||
-      (st = upload(p->tdiag_d, tdiag.data(), nbar, s)) || (st = upload(p->tup_d, tup.data(), nbar, s)) ||
-      (st = upload(p->tlo_f, flo.data(), nbar, s)) || (st = upload(p->tdiag_f, fdiag.data(), nbar, s)) ||
-      (st = upload(p->tup_f, fup.data(), nbar, s)) || (st = upload(p->xlo, h.xlo.data(), p->nrx, s)) ||
-      (st = upload(p->xdiag, h.xdiag.data(), p->nrx, s)) || (st = upload(p->xup, h.xup.data(), p->nrx, s)) ||
-      (st = upload(p->rxl, rxl.data(), p->nrx, s)) || (st = upload(p->rxd, rxd.data(), p->nrx, s)) ||
-      (st = upload(p->rxu, rxu.data(), p->nrx, s)))
-    return st;
-  std::vector<double> rdd(p->dim == 2 ? p->nbar : 0);
-  if (p->dim == 2)  // row iy of the stacked grid belongs to problem iy / nym (its x-coefficients)
-    for (int64_t iy = 0; iy < p->ny; ++iy)
-      for (int64_t x = 0; x < p->nx; ++x) rdd[iy * p->nx + x] = rxd[(iy / p->nym) * p->nx + x] + ryd[iy];
-  if (p->dim == 2 && ((st = upload(p->rdd, rdd.data(), p->nbar, s)) ||
-                      (st = upload(p->ryl, ryl.data(), p->ny, s)) || (st = upload(p->ryd, ryd.data(), p->ny, s)) ||
-                      (st = upload(p->ryu, ryu.data(), p->ny, s)) || (st = upload(p->ylo, h.ylo.data(), p->ny, s)) ||
-                      (st = upload(p->ydiag, h.ydiag.data(), p->ny, s)) || (st = upload(p->yup, h.yup.data(), p->ny, s))))
-    return st;
+  p->hop.clear();
+  for (const auto *v : {&h.xlo, &h.xdiag, &h.xup}) p->hop.insert(p->hop.end(), v->begin(), v->end());
+  if (p->dim == 2)
+    for (const auto *v : {&h.ylo, &h.ydiag, &h.yup, &h.mu}) p->hop.insert(p->hop.end(), v->begin(), v->end());
+  if ((st = upload(p->opsrc, p->hop.data(), p->hop.size(), s))) return st;
+  pd::OperatorArgs o{};
+  o.nbar = p->nbar;
+  o.nrx = p->nrx;
+  o.ny = p->ny;
+  o.nx = p->nx;
+  o.nym = p->nym;
+  o.tau = p->tau;
+  o.xlo = p->opsrc;
+  o.xdiag = o.xlo + p->nrx;
+  o.xup = o.xdiag + p->nrx;
+  if (p->dim == 2) {
+    o.ylo = o.xup + p->nrx;
+    o.ydiag = o.ylo + p->ny;
+    o.yup = o.ydiag + p->ny;
+    o.mu = o.yup + p->ny;
+  }
+  o.klo = p->klo;
+  o.kdiag = p->kdiag;
+  o.kup = p->kup;
+  o.tlo_d = p->tlo_d;
+  o.tdiag_d = p->tdiag_d;
+  o.tup_d = p->tup_d;
+  o.tlo_f = p->tlo_f;
+  o.tdiag_f = p->tdiag_f;
+  o.tup_f = p->tup_f;
+  o.rxl = p->rxl;
+  o.rxd = p->rxd;
+  o.rxu = p->rxu;
+  o.ryl = p->ryl;
+  o.ryd = p->ryd;
+  o.ryu = p->ryu;
+  o.rdd = p->rdd;
+  pd::launch_operator(p->ctx, o);
   if (p->batch > 1) {
-    std::vector<int> bnx(p->batch);
     // unknowns of problem b inside its slot (2D: the whole nx x ny grid)
+    p->hbnx.resize(p->batch);
     for (int b = 0; b < p->batch; ++b)
-      bnx[b] = p->dim == 2 ? (int)p->nxm : (int)(desc->batch_nx ? desc->batch_nx[b] : desc->nx);
-    if ((st = upload(p->bnx, bnx.data(), p->batch, s))) return st;
+      p->hbnx[b] = p->dim == 2 ? (int)p->nxm : (int)(desc->batch_nx ? desc->batch_nx[b] : desc->nx);
+    if ((st = upload(p->bnx, p->hbnx.data(), p->batch, s))) return st;
   }
-  std::vector<double> msc;
   if (p->mass) {  // M^{-1/2}; identity when the descriptor carries no mass matrix
-    msc.assign(nbar, 1.0);
+    p->hmsc.assign(p->nbar, 1.0);
     if (desc->m_diag)
-      for (int64_t j = 0; j < nbar; ++j) msc[j] = 1.0 / std::sqrt(desc->m_diag[j]);
-    if ((st = upload(p->msc, msc.data(), nbar, s))) return st;
+      for (int64_t j = 0; j < p->nbar; ++j) p->hmsc[j] = 1.0 / std::sqrt(desc->m_diag[j]);
+    if ((st = upload(p->msc, p->hmsc.data(), p->nbar, s))) return st;
   }
-  // the host vectors die on return: wait for the copies
-  if (cudaStreamSynchronize(s) != cudaSuccess) return fail(PD_ERR_CUDA, "operator upload failed");
-  return PD_OK;
+  return ctx_status(p);
 }
 
 pd_status ctx_status(pd_plan *p) {
@@ -1862,18 +1852,17 @@ pd_status paradiag_set_operator(pd_plan *p, const pd_desc *desc) {
   if (desc->m_diag && !p->mass)
     return fail(PD_ERR_INVALID_ARG, "paradiag_set_operator: the plan was built without a mass matrix");
   if (batch == 1 && desc->tau != p->tau) {  // tau reaches some kernels by value: re-capture
-    if (p->ctx.stream) cudaStreamSynchronize(p->ctx.stream);
+    cudaStreamSynchronize(p->ctx.stream);
     drop_graph(p);
     p->tau = desc->tau;
   }
-  if (p->ctx.stream) cudaStreamSynchronize(p->ctx.stream);  // no solve may still read the old operator
+  cudaStreamSynchronize(p->ctx.stream);  // no solve may still read the old operator, no upload its host side
   std::lock_guard<std::recursive_mutex> lk(host_mutex());
   const bool lane_before = p->lane;
   if ((st = upload_operator(p, desc)) != PD_OK) return st;
   if (p->lane != lane_before) drop_graph(p);  // the lane's arguments are captured in the graph
   if ((st = factorize(p)) != PD_OK) return st;
-  if (p->ctx.stream && cudaStreamSynchronize(p->ctx.stream) != cudaSuccess)
-    return fail(PD_ERR_CUDA, "operator factorisation failed");
+  if (cudaStreamSynchronize(p->ctx.stream) != cudaSuccess) return fail(PD_ERR_CUDA, "operator upload failed");
   return PD_OK;
 }
 
