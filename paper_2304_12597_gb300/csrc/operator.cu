@@ -38,6 +38,12 @@ __global__ void __launch_bounds__(256) k_operator(OperatorArgs o) {
     o.tlo_f[j] = (float)tl;
     o.tdiag_f[j] = (float)td;
     o.tup_f[j] = (float)tu;
+    // T_x's row sum first (exact zeros stay zero), then the mode's eigenvalue; the couplings out
+    // of a block do not exist
+    const int64_t ix = j % o.nx;
+    const double sl = ix > 0 ? lo : 0.0, su = ix + 1 < o.nx ? up : 0.0;
+    const double e = (o.xdiag[i] + sl) + su;
+    o.texc_f[j] = (float)(o.tau * (o.mu ? e + o.mu[r] : e));
   }
   if (o.mu) o.rdd[j] = fma(o.tau, o.xdiag[i], 1.0) + o.tau * o.ydiag[r];
 }

@@ -220,6 +220,7 @@ struct OperatorArgs {
   double *klo, *kdiag, *kup;                    // K in the solve basis (nbar)
   double *tlo_d, *tdiag_d, *tup_d;              // tau K
   float *tlo_f, *tdiag_f, *tup_f;               // the same in binary32, or null
+  float *texc_f;                                // tau times the row sums of K, formed in FP64
   double *rxl, *rxd, *rxu, *ryl, *ryd, *ryu, *rdd;  // residual coefficients
 };
 void launch_operator(Ctx &c, const OperatorArgs &o);
@@ -261,6 +262,7 @@ struct PintArgs {
   const cpx<T> *shift_t;   // the same in the compute type (binary32 plans; null = convert)
   const cpx<T> *omega_t;   // omega in the compute type (null = convert)
   const T *tlo, *tdiag, *tup;  // tau * K (block-decoupled), length nblk*blen
+  const T *texc;           // tau times the row sums of K within a block (k_pint_chunk's diagonal)
   const cpx<T> *R;         // spectrum right-hand sides (nf, ldr) or null
   int64_t ldr;
   const T *rvec;           // real vector: the right-hand side when R is null,

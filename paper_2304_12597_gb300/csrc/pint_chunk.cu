@@ -5,12 +5,27 @@
 // One team of P lanes solves one tridiagonal block of blen <= P M rows; lane t owns the M
 // consecutive rows from t M in registers.
 //  1. Forward: rows 0..M-2 of the chunk become x_i + aa_i X + cc_i x_{i+1} = r_i, where X is the
-//     last unknown of the chunk before.
-//  2. Backward (scalars only): x_0 = D - A X - C L, where L is the chunk's own last unknown.
-//  3. Row M-1 and the next chunk's x_0 give one row in (X, L, next L) per chunk: P rows, solved by
+//     last unknown of the chunk before; beside it, x_0 = D - A X + w L with the chunk's own last
+//     unknown L.
+//  2. Row M-1 and the next chunk's x_0 give one row in (X, L, next L) per chunk: P rows, solved by
 //     parallel cyclic reduction on unit-diagonal rows (P <= 32: shuffles; wider teams: shared memory).
-//  4. Back substitution from L: x_i = r_i - aa_i X - cc_i x_{i+1}.
+//  3. Back substitution from L: x_i = r_i - aa_i X - cc_i x_{i+1}.
 // Elimination is without pivoting inside principal blocks, as in pint.cu.
+//
+// Every row carries its excess, the sum of its coefficients, instead of its diagonal: a pivot is
+// then excess - (off-diagonals), and the excess itself is updated by row operations of its own.
+// For M-matrices (heat, upwinding: off-diagonals <= 0, excess >= 0) all these are sums of terms
+// of one sign (with a complex shift: terms within a quarter plane), so pivots lose nothing to
+// cancellation, however ill-conditioned the small shifts make the system (A. K. Alfa, J. Xue,
+// Q. Ye, Math. Comp. 71 (2002): elimination of diagonally dominant M-matrices from their
+// off-diagonals and row sums).  With the diagonal instead, 1 - lo up / pivot cancels to the
+// row's small excess and a binary32 solve of the low frequencies is off by kappa u: 2e-4 on
+// 1023 x 1024 heat, against 1e-5 this way, and the sum tau (lo + diag + up) no longer depends on
+// the rounding of the three coefficients to binary32.  The refinement then contracts by 1e-5 to
+// 1e-6 a sweep instead of 1e-3 to 1e-4, at about 25 % more arithmetic in this kernel (2D: 43 -> 44 us
+// per loop): advdiff1d_4095x2048 and heat2d_255x255x256 take 3 solves instead of 4 (1530 ->
+// 1160 us, 2964 -> 2234 us), 32 x heat1d_1023x1024 takes 3 instead of 5 (5336 -> 3297 us).
+// For other signs the same identities hold, with the rounding of a dominant elimination.
 //
 // What bounds it: instruction issue.  Against k_pint's two separators per chunk of 8 rows held
 // in shared memory this takes 16 rows per lane (half the PCR levels per row), keeps aa, cc, r
@@ -45,6 +60,7 @@ using C = cpx<float>;
 __device__ __forceinline__ C nmul(C a, C b) {
   return mk<float>(fmaf(a.y, b.y, -(a.x * b.x)), -fmaf(a.x, b.y, a.y * b.x));
 }
+__device__ __forceinline__ C sub1(C a, float s) { return mk<float>(a.x - s, a.y); }
 __device__ __forceinline__ C shfl_up(C v, int d, int w) {
   return mk<float>(__shfl_up_sync(0xffffffffu, v.x, d, w), __shfl_up_sync(0xffffffffu, v.y, d, w));
 }
@@ -52,20 +68,26 @@ __device__ __forceinline__ C shfl_dn(C v, int d, int w) {
   return mk<float>(__shfl_down_sync(0xffffffffu, v.x, d, w), __shfl_down_sync(0xffffffffu, v.y, d, w));
 }
 
-// One PCR level on unit-diagonal rows a x_lo + x + c x_hi = d, given the neighbours' rows.
-// A row without a lower (upper) neighbour has a = 0 (c = 0), so whatever finite row stands in
-// for the missing neighbour drops out.
-__device__ __forceinline__ void pcr_level(C &a, C &c, C &d, C al, C cl, C dl, C ah, C ch, C dh, bool last) {
-  C den = mk<float>(1.0f, 0.0f);
-  den = fnms(den, a, cl);
-  den = fnms(den, c, ah);
-  const C r = recip(den);
-  const C nd = mul(fnms(fnms(d, a, dl), c, dh), r);
+__device__ __forceinline__ C fma_c(C a, C b, C c) {  // a + b c
+  return mk<float>(fmaf(-b.y, c.y, fmaf(b.x, c.x, a.x)), fmaf(b.y, c.x, fmaf(b.x, c.y, a.y)));
+}
+
+// A unit-diagonal row a x_lo + x + c x_hi = d with its excess g = 1 + a + c carried beside it.
+struct SepRow {
+  C a, c, d, g;
+};
+// One PCR level, given the neighbours' rows.  A row without a lower (upper) neighbour has a = 0
+// (c = 0), so whatever finite row stands in for the missing neighbour drops out.
+__device__ __forceinline__ void pcr_level(SepRow &r, const SepRow &l, const SepRow &h, bool last) {
+  const C a = nmul(r.a, l.a), c = nmul(r.c, h.c);
+  const C g = fnms(fnms(r.g, r.a, l.g), r.c, h.g);
+  const C q = recip(sub(sub(g, a), c));
+  r.d = mul(fnms(fnms(r.d, r.a, l.d), r.c, h.d), q);
   if (!last) {
-    a = mul(nmul(a, al), r);
-    c = mul(nmul(c, ch), r);
+    r.a = mul(a, q);
+    r.c = mul(c, q);
+    r.g = mul(g, q);
   }
-  d = nd;
 }
 
 }  // namespace
@@ -91,7 +113,7 @@ __global__ void __launch_bounds__(NT, MINB) k_pint_chunk(PintGeom g, PintArgs<fl
   const int64_t off = (int64_t)blk * blen;
 
   extern __shared__ __align__(16) unsigned char smraw[];
-  float4 *cs = reinterpret_cast<float4 *>(smraw);                // tau lo, tau diag, tau up, vector
+  float4 *cs = reinterpret_cast<float4 *>(smraw);                // tau lo, tau (lo + diag + up), tau up, vector
   constexpr int NB = NT >= 256 ? 1 : 2;                          // right-hand-side buffers
   C *bufs = reinterpret_cast<C *>(cs + TS);                      // [NB][teams][TS]
   double2 *red = reinterpret_cast<double2 *>(bufs + (size_t)NB * teams * TS);  // PW == 0: [warps][mdots]
@@ -161,7 +183,7 @@ __global__ void __launch_bounds__(NT, MINB) k_pint_chunk(PintGeom g, PintArgs<fl
         const bool in = e < blen;
         // rows outside the block do not exist: its first lo and last up are zero
         q[u].x = in && e > 0 ? a.tlo[off + e] : 0.0f;
-        q[u].y = in ? a.tdiag[off + e] : 1.0f;
+        q[u].y = in ? a.texc[off + e] : 1.0f;
         q[u].z = in && e + 1 < blen ? a.tup[off + e] : 0.0f;
         q[u].w = in && rvec && !xy ? rvec[off + e] : 0.0f;
       }
@@ -222,9 +244,10 @@ __global__ void __launch_bounds__(NT, MINB) k_pint_chunk(PintGeom g, PintArgs<fl
     const C s = a.shift_t[live ? k : 0];
     C *my = buf + t * (M + 1);
 
-    // 1. forward elimination
+    // 1. forward: row i as (aa, 1, cc), its excess gg, and x_0 = D - A X + w x_{i+1} with the
+    // excess gm = 1 + A - w
     C aa[M], cc[M], r[M];
-    C sep_a, sep_b, sep_d;
+    C D, A, w, gm, gg, sep_a, sep_g, sep_d;
     float sep_up;
 #pragma unroll
     for (int i = 0; i < M; ++i) {
@@ -232,81 +255,81 @@ __global__ void __launch_bounds__(NT, MINB) k_pint_chunk(PintGeom g, PintArgs<fl
       C ri = has_r ? my[i] : mk<float>(q.w, 0.0f);
       if (has_r) ri.x -= q.w;
       // rows past the block's end: 1 x = 0, whatever the shift
-      const C d = (tail && t * M + i >= blen) ? mk<float>(1.0f, 0.0f) : mk<float>(s.x + q.y, s.y);
-      if (i == 0) {
-        const C rd = recip(d);
-        aa[0] = scal(q.x, rd);
-        cc[0] = scal(q.z, rd);
-        r[0] = mul(ri, rd);
-      } else if (i < M - 1) {
-        const C rd = recip(fnms_r(d, q.x, cc[i - 1]));
-        const C lr = scal(q.x, rd);
-        aa[i] = nmul(lr, aa[i - 1]);
+      const C e = (tail && t * M + i >= blen) ? mk<float>(1.0f, 0.0f) : mk<float>(s.x + q.y, s.y);
+      const C al = i == 0 ? mk<float>(q.x, 0.0f) : scal(-q.x, aa[i - 1]);
+      const C g1 = i == 0 ? e : fnms_r(e, q.x, gg);
+      if (i > 0) ri = fnms_r(ri, q.x, r[i - 1]);
+      if (i < M - 1) {
+        const C rd = recip(sub1(sub(g1, al), q.z));
+        aa[i] = i == 0 ? scal(q.x, rd) : mul(al, rd);
         cc[i] = scal(q.z, rd);
-        r[i] = mul(fnms_r(ri, q.x, r[i - 1]), rd);
+        gg = mul(g1, rd);
+        r[i] = mul(ri, rd);
+        D = i == 0 ? r[0] : fma_c(D, w, r[i]);
+        A = i == 0 ? aa[0] : fma_c(A, w, aa[i]);
+        gm = i == 0 ? gg : fma_c(gm, w, gg);
+        w = i == 0 ? scal(-1.0f, cc[0]) : nmul(w, cc[i]);
       } else {
-        sep_a = scal(-q.x, aa[M - 2]);
-        sep_b = fnms_r(d, q.x, cc[M - 2]);
-        sep_d = fnms_r(ri, q.x, r[M - 2]);
+        sep_a = al;
+        sep_g = g1;
+        sep_d = ri;
         sep_up = q.z;
       }
     }
-    // 2. x_0 = D - A X - C L
-    C A = aa[M - 2], Cc = cc[M - 2], D = r[M - 2];
-#pragma unroll
-    for (int i = M - 3; i >= 0; --i) {
-      D = fnms(r[i], cc[i], D);
-      A = fnms(aa[i], cc[i], A);
-      Cc = nmul(cc[i], Cc);
-    }
-    // 3. one row per chunk in (X, L, next L), unit diagonal, and its PCR
+    // 2. one row per chunk in (X, L, next L), unit diagonal, and its PCR
+    auto sep_row = [&](C An, C wn, C gn, C Dn) {
+      SepRow v;
+      v.a = sep_a;
+      v.c = scal(sep_up, wn);
+      v.g = fnms_r(sep_g, sep_up, gn);
+      const C q = recip(sub(sub(v.g, v.a), v.c));
+      v.a = mul(v.a, q);
+      v.c = mul(v.c, q);
+      v.g = mul(v.g, q);
+      v.d = mul(fnms_r(sep_d, sep_up, Dn), q);
+      return v;
+    };
     C L, X;
     if constexpr (PW != 0) {
-      const C An = shfl_dn(A, 1, PW), Cn = shfl_dn(Cc, 1, PW), Dn = shfl_dn(D, 1, PW);
-      const C rb = recip(fnms_r(sep_b, sep_up, An));
-      C ra = mul(sep_a, rb);
-      C rc = mul(scal(-sep_up, Cn), rb);
-      C rd = mul(fnms_r(sep_d, sep_up, Dn), rb);
+      SepRow v = sep_row(A, shfl_dn(w, 1, PW), shfl_dn(gm, 1, PW), shfl_dn(D, 1, PW));
 #pragma unroll
       for (int sg = 1; sg < PW; sg <<= 1) {
-        const C al = shfl_up(ra, sg, PW), cl = shfl_up(rc, sg, PW), dl = shfl_up(rd, sg, PW);
-        const C ah = shfl_dn(ra, sg, PW), ch = shfl_dn(rc, sg, PW), dh = shfl_dn(rd, sg, PW);
-        pcr_level(ra, rc, rd, al, cl, dl, ah, ch, dh, 2 * sg >= PW);
+        const SepRow lo{shfl_up(v.a, sg, PW), shfl_up(v.c, sg, PW), shfl_up(v.d, sg, PW), shfl_up(v.g, sg, PW)};
+        const SepRow hi{shfl_dn(v.a, sg, PW), shfl_dn(v.c, sg, PW), shfl_dn(v.d, sg, PW), shfl_dn(v.g, sg, PW)};
+        pcr_level(v, lo, hi, 2 * sg >= PW);
       }
-      L = rd;
+      L = v.d;
       X = shfl_up(L, 1, PW);
       if (t == 0) X = mk<float>(0.0f, 0.0f);
     } else {
       // the exchanged rows sit in the lanes' own chunk slots of the buffer, which each lane has
-      // read by now: six slots of a lane, in two triples that alternate.  A triple is rewritten
-      // two levels later, past the barrier that every lane reaches after reading it.
-      my[0] = A;
-      my[1] = Cc;
-      my[2] = D;
+      // read by now: eight slots of a lane, in two sets of four that alternate.  A set is
+      // rewritten two levels later, past the barrier that every lane reaches after reading it.
+      my[0] = D;
+      my[1] = w;
+      my[2] = gm;
       __syncthreads();
       const C *nx = my + (t + 1 < P ? M + 1 : 0);
-      const C rb = recip(fnms_r(sep_b, sep_up, nx[0]));
-      C ra = mul(sep_a, rb);
-      C rc = mul(scal(-sep_up, nx[1]), rb);
-      C rd = mul(fnms_r(sep_d, sep_up, nx[2]), rb);
-      int lv = 3;
-      for (int sg = 1; sg < P; sg <<= 1, lv ^= 3) {
+      SepRow v = sep_row(A, nx[1], nx[2], nx[0]);
+      int lv = 4;
+      for (int sg = 1; sg < P; sg <<= 1, lv ^= 4) {
         C *own = my + lv;
-        own[0] = ra;
-        own[1] = rc;
-        own[2] = rd;
+        own[0] = v.a;
+        own[1] = v.c;
+        own[2] = v.d;
+        own[3] = v.g;
         __syncthreads();
         const C *lo = own - (t >= sg ? sg * (M + 1) : 0), *hi = own + (t + sg < P ? sg * (M + 1) : 0);
-        pcr_level(ra, rc, rd, lo[0], lo[1], lo[2], hi[0], hi[1], hi[2], 2 * sg >= P);
+        pcr_level(v, SepRow{lo[0], lo[1], lo[2], lo[3]}, SepRow{hi[0], hi[1], hi[2], hi[3]}, 2 * sg >= P);
       }
-      L = rd;
+      L = v.d;
       my[lv] = L;
       __syncthreads();
       X = t > 0 ? my[lv - (M + 1)] : mk<float>(0.0f, 0.0f);
       __syncthreads();  // x goes into the slots next
     }
 
-    // 4. back substitution, and the accumulation of b (eq. 7)
+    // 3. back substitution, and the accumulation of b (eq. 7)
     float ox = 0.0f, oy = 0.0f;
     if (MODE == kAcc && live) {
       if (a.omega_t) {
@@ -327,7 +350,7 @@ __global__ void __launch_bounds__(NT, MINB) k_pint_chunk(PintGeom g, PintArgs<fl
     }
     if (out) sync_team();
 
-    // 5. store
+    // 4. store
     if (a.Y) {
 #pragma unroll
       for (int j = 0; j < M; ++j) {
@@ -344,7 +367,7 @@ __global__ void __launch_bounds__(NT, MINB) k_pint_chunk(PintGeom g, PintArgs<fl
           a.Y[(int64_t)(kb + q) * a.ldy + off + e] = bufs[((size_t)b * teams + q) * TS + e + e / M];
       }
     }
-    // 6. g_k = V_m^T y_k: sums over a warp in binary32, over a team's warps in FP64
+    // 5. g_k = V_m^T y_k: sums over a warp in binary32, over a team's warps in FP64
     if (MODE == kDots && mdots > 0) {
       C yv[M];
 #pragma unroll

@@ -256,7 +256,7 @@ struct pd_plan {
   float *ts_f = nullptr, *tsi_f = nullptr;
   double *klo = nullptr, *kdiag = nullptr, *kup = nullptr;
   double *tlo_d = nullptr, *tdiag_d = nullptr, *tup_d = nullptr;
-  float *tlo_f = nullptr, *tdiag_f = nullptr, *tup_f = nullptr;
+  float *tlo_f = nullptr, *tdiag_f = nullptr, *tup_f = nullptr, *texc_f = nullptr;
   // compact source of the operator: T_x (lo, diag, up; nrx each), 2D: T_y (lo, diag, up) and the
   // modes' eigenvalues (ny each); hop and hmsc, hbnx are the host sides of its uploads
   double *opsrc = nullptr;
@@ -521,9 +521,8 @@ void fill_geometry(pd_plan *p, const pd_desc *d) {
   p->precision = d->precision;
   p->maxit = d->maxit ? d->maxit : 32;
   p->q = d->q > 1 ? d->q : 1;
-  // PD_MIXED: a binary32 solve is accurate to ~1e-4 whatever Algorithm 2 does past that
-  // (measured: tighter tolerances add Krylov steps, not accuracy), so the first solve's
-  // Algorithm 2 stops at 1e-4; refinement does the rest
+  // PD_MIXED: the first solve's Algorithm 2 stops at 1e-4 (tighter tolerances add Krylov
+  // steps and do not save a refinement sweep); refinement does the rest
   p->eps = d->eps_krylov > 0 ? d->eps_krylov : (d->precision == PD_FP64 ? 1e-13 : 1e-4);
   // FP64 plans that refine anyway use a loose tolerance per solve: Algorithm 3 loses
   // up to kappa(F D_alpha) per solve, and a batch runs until its slowest problem's
@@ -669,6 +668,7 @@ size_t layout(pd_plan *p, unsigned char *base) {
     p->tlo_f = A.take<float>(nbar);
     p->tdiag_f = A.take<float>(nbar);
     p->tup_f = A.take<float>(nbar);
+    p->texc_f = A.take<float>(nbar);
   }
   p->opsrc = A.take<double>(3 * p->nrx + (p->dim == 2 ? 4 * p->ny : 0));
   p->rxl = A.take<double>(p->nrx);
@@ -947,7 +947,7 @@ pd_status upload_operator(pd_plan *p, const pd_desc *desc) {
   o.nbar = p->nbar;
   o.nrx = p->nrx;
   o.ny = p->ny;
-  o.nx = p->nx;
+  o.nx = p->blen;
   o.nym = p->nym;
   o.tau = p->tau;
   o.xlo = p->opsrc;
@@ -968,6 +968,7 @@ pd_status upload_operator(pd_plan *p, const pd_desc *desc) {
   o.tlo_f = p->tlo_f;
   o.tdiag_f = p->tdiag_f;
   o.tup_f = p->tup_f;
+  o.texc_f = p->texc_f;
   o.rxl = p->rxl;
   o.rxd = p->rxd;
   o.rxu = p->rxu;
@@ -1070,6 +1071,7 @@ pd::PintArgs<float> base_args<float>(pd_plan *p) {
   a.tlo = p->tlo_f;
   a.tdiag = p->tdiag_f;
   a.tup = p->tup_f;
+  a.texc = p->texc_f;
   // the zero frequency, whose shifted system carries the ill-conditioning of tau K, in FP64
   a.k0_fp64 = p->lane ? 1 : 0;
   a.tlo_d = p->tlo_d;
@@ -1141,8 +1143,8 @@ pd::KrylovBufs kbufs(pd_plan *p) {
 // the eq. (13) residual stops halving near the precision floor: in binary32 it
 // levels off at the rounding noise of the shifted solves, and in FP64 the polynomial
 // space K_m(K, b) can stall for many steps when J_l is far from I.  A binary32
-// refinement sweep contracts the error by ~1e-3 at best (rounding noise of the
-// residual, amplified by the solution operator), so its Algorithm 2 asks for 1e-3; FOM
+// refinement sweep contracts the error by 1e-3 (k_pint) to 1e-5 (k_pint_chunk), and what
+// its Algorithm 2 leaves is corrected by the next one, so it asks for 3e-3; FOM
 // residuals are not monotone, so it leaves on a stall only after two checks without
 // halving and once ||r_m|| <= 1e-2 ref (far above the binary32 noise floor of eq. 13, far
 // below a residual that would keep the refinement from contracting).  FP64 refinement
