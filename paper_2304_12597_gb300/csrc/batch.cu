@@ -53,16 +53,6 @@ __global__ void k_batch_exponents(int batch, int nc, const double *__restrict__ 
   zero[b] = s == 0.0 ? 1 : 0;
 }
 
-// x * 2^k exactly: an exponent-field add for normal x whose result stays normal
-// (zero stays zero); other cases (subnormal, overflow, Inf/NaN) take ldexp.
-__device__ __forceinline__ double pow2_scale(double x, int k) {
-  const long long bits = __double_as_longlong(x);
-  if ((bits & 0x7fffffffffffffffLL) == 0) return x;
-  const int e = (int)((bits >> 52) & 0x7ff);
-  if (e > 0 && e < 0x7ff && e + k > 0 && e + k < 0x7ff) return __longlong_as_double(bits + ((long long)k << 52));
-  return ldexp(x, k);
-}
-
 // Y = X * 2^(sign * ex[slot]) over the (nt, ld) array, one time row per blockIdx.y;
 // Y may alias X.  With nxb != NULL, columns past problem b's n_x, and every column of an
 // all-zero problem (zero[b]), are set to zero (they are decoupled from the problem, but

@@ -13,6 +13,7 @@
 #include <algorithm>
 
 #include "pd_control.cuh"
+#include "pd_fft.cuh"
 
 namespace pd {
 
@@ -176,54 +177,6 @@ __host__ __device__ inline int pz(int i) { return i + (i >> 4); }
 __host__ __device__ inline int series_stride16(int n) {
   const int s0 = n + n / 16;
   return s0 + (((2 - s0) % 16) + 16) % 16;
-}
-
-// X[k] = sum_i x[i] w^{ik}, w = exp(-2 pi i / 16), in place, natural order in and out:
-// radix-4 over i = 4 i1 + i2 (i1 first), twiddles w^{i2 k1}, radix-4 over i2.
-template <typename T>
-__device__ __forceinline__ void radix4_fwd(cpx<T> &a0, cpx<T> &a1, cpx<T> &a2, cpx<T> &a3) {
-  const cpx<T> t0 = add(a0, a2), t1 = sub(a0, a2), t2 = add(a1, a3), t3 = sub(a1, a3);
-  const cpx<T> mt3 = mk<T>(t3.y, -t3.x);  // -i t3
-  a0 = add(t0, t2);
-  a2 = sub(t0, t2);
-  a1 = add(t1, mt3);
-  a3 = sub(t1, mt3);
-}
-template <typename T>
-__device__ __forceinline__ cpx<T> w16(int m) {  // w^m for the products m of i2, k1 < 4
-  constexpr double c = 0.92387953251128675613;  // cos(pi/8)
-  constexpr double s = 0.38268343236508977173;  // sin(pi/8)
-  constexpr double r = 0.70710678118654752440;  // cos(pi/4)
-  switch (m) {
-    case 1: return mk<T>((T)c, (T)-s);
-    case 2: return mk<T>((T)r, (T)-r);
-    case 3: return mk<T>((T)s, (T)-c);
-    case 4: return mk<T>(T(0), T(-1));
-    case 6: return mk<T>((T)-r, (T)-r);
-    case 9: return mk<T>((T)-c, (T)s);
-    default: return mk<T>(T(1), T(0));
-  }
-}
-template <typename T>
-__device__ __forceinline__ void dft16(cpx<T> (&x)[16]) {
-#pragma unroll
-  for (int i2 = 0; i2 < 4; ++i2) radix4_fwd(x[i2], x[4 + i2], x[8 + i2], x[12 + i2]);  // x[4 k1 + i2]
-#pragma unroll
-  for (int k1 = 1; k1 < 4; ++k1)
-#pragma unroll
-    for (int i2 = 1; i2 < 4; ++i2) x[4 * k1 + i2] = mul(w16<T>(i2 * k1), x[4 * k1 + i2]);
-  cpx<T> y[16];
-#pragma unroll
-  for (int k1 = 0; k1 < 4; ++k1) {
-    cpx<T> b0 = x[4 * k1], b1 = x[4 * k1 + 1], b2 = x[4 * k1 + 2], b3 = x[4 * k1 + 3];
-    radix4_fwd(b0, b1, b2, b3);
-    y[k1] = b0;
-    y[k1 + 4] = b1;
-    y[k1 + 8] = b2;
-    y[k1 + 12] = b3;
-  }
-#pragma unroll
-  for (int k = 0; k < 16; ++k) x[k] = y[k];
 }
 
 // The DIT stages of half-span 16 and up (the radix-16 first stage done), on series held
@@ -617,19 +570,6 @@ __global__ void __launch_bounds__(256) k_fft_c2r(const cpx<T> *__restrict__ S, i
   }
 }
 
-// The FP64 all-at-once residual as the DST's input (ResIn.G != null): element (row y, column
-// col) of slab s (time t = s / batch, problem b = s % batch) is
-// r = G_t + u_{t-1} - [(I + tau T_x) u_t + tau T_y u_t] at row b nym + y of the stacked grid
-// (ny = batch nym rows, x-coefficients of problem b), times 2^mex[b] for batches: five
-// FMAs in FP64 per element after G_t + u_{t-1} (the diagonal 1 + tau (d_x + d_y) comes
-// precombined per grid point in rdd), formed while the DST loads its tile.
-struct ResIn {
-  const double *G, *U;
-  const double *rxl, *rdd, *rxu, *ryl, *ryu;
-  int ny, nym, batch;
-  const int *mex;
-};
-
 // Orthonormal DST-I along y via a length N = 2(ny+1) complex FFT of the odd
 // extension, two x-columns packed per series (a + i b):
 //   DST_l(a) = -Im Z[l] / 2,  DST_l(b) = Re Z[l] / 2,  scaled by sqrt(2/(ny+1)).
@@ -913,6 +853,9 @@ void launch_fft_c2r(Ctx &c, const cpx<T> *S, int64_t lds, int64_t ncols, int n, 
 template <typename Tin, typename Tout, typename T, bool RES>
 static void dst_launch(Ctx &c, const Tin *X, Tout *Y, int64_t nslab, int64_t ny, int64_t nx, const cpx<T> *tw,
                        int mode, const int *skip, const ResIn &rin, const char *fam, double bytes) {
+  // the half-extension kernel where it is the faster one, unless the caller chose a first-stage radix
+  if (c.fft_radix == 0 && dst2_fits(ny, nslab * nx, RES && sizeof(T) == 4))
+    return launch_dst2<Tin, Tout, T, RES>(c, X, Y, nslab * nx, ny, nx, tw, mode, skip, rin, fam, bytes);
   const int N = (int)(2 * (ny + 1));
   const int logN = ilog2(N);
   const int TX = pick_tx<T>(c, N, sizeof(T) == 8 ? 8 : 16, nslab * nx);

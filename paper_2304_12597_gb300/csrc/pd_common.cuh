@@ -92,8 +92,7 @@ __device__ __forceinline__ void team_sync(int P, int team_in_cta) {
 // arithmetic, such as the residual, this frees the FP64 pipe; measured 8% on the 2D residual
 // DST).  The significand is truncated (error below one binary32 ulp, where round-to-nearest
 // gives half an ulp); magnitudes below binary32's normal range become zero, above it
-// infinity; NaN stays NaN.  binary32 -> binary64 keeps the hardware conversion, which
-// measured faster than its integer form.
+// infinity; NaN stays NaN.
 __device__ __forceinline__ float f64_to_f32_bits(double x) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
   const unsigned hi = (unsigned)(b >> 32), lo = (unsigned)b;
@@ -110,13 +109,35 @@ __device__ __forceinline__ float f64_to_f32_bits(double x) {
   }
   return __uint_as_float(r);
 }
-// cvt<To>(x): x in type To, binary64 -> binary32 through the integer conversion above.
+// binary32 -> binary64 by integer operations, for the same reason (the stores of the inverse
+// transforms: one conversion beside the one FP64 add of U += delta).  Exact for normal numbers
+// and infinities; subnormals become zero, NaN stays NaN.
+__device__ __forceinline__ double f32_to_f64_bits(float x) {
+  const unsigned b = __float_as_uint(x), m = b & 0x7fffffffu;
+  unsigned hi = (m >> 3) + (m >= 0x7f800000u ? 0x70000000u : 0x38000000u);  // exponent + 896 (+ 1792)
+  unsigned lo = m << 29;
+  if (m < 0x00800000u) hi = lo = 0u;
+  return __hiloint2double((int)(hi | (b & 0x80000000u)), (int)lo);
+}
+// cvt<To>(x): x in type To, between binary64 and binary32 through the integer conversions above.
 template <typename To, typename From>
 __device__ __forceinline__ To cvt(From x) {
   if constexpr (sizeof(To) == 4 && sizeof(From) == 8)
     return f64_to_f32_bits(x);
+  else if constexpr (sizeof(To) == 8 && sizeof(From) == 4)
+    return f32_to_f64_bits(x);
   else
     return (To)x;
+}
+
+// x * 2^k exactly: an exponent-field add for normal x whose result stays normal
+// (zero stays zero); other cases (subnormal, overflow, Inf/NaN) take ldexp.
+__device__ __forceinline__ double pow2_scale(double x, int k) {
+  const long long bits = __double_as_longlong(x);
+  if ((bits & 0x7fffffffffffffffLL) == 0) return x;
+  const int e = (int)((bits >> 52) & 0x7ff);
+  if (e > 0 && e < 0x7ff && e + k > 0 && e + k < 0x7ff) return __longlong_as_double(bits + ((long long)k << 52));
+  return ldexp(x, k);
 }
 
 // Programmatic dependent launch: every kernel of this library opens with this wait,

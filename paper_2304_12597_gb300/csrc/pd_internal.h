@@ -196,6 +196,25 @@ void launch_fft_c2r(Ctx &c, const cpx<T> *S, int64_t lds, int64_t ncols, int n, 
                     void *out, int64_t ldo, int mode, double *norm_part, int *nparts,
                     const StepFinish *fin = nullptr, const T *rsi = nullptr, double *colsum = nullptr,
                     const int *mex = nullptr, int mnx = 1, const int *skip = nullptr);
+// The FP64 all-at-once residual as the DST's input (ResIn.G != null): element (row y, column
+// col) of slab s (time t = s / batch, problem b = s % batch) is
+// r = G_t + u_{t-1} - [(I + tau T_x) u_t + tau T_y u_t] at row b nym + y of the stacked grid
+// (ny = batch nym rows, x-coefficients of problem b), times 2^mex[b] for batches: five
+// FMAs in FP64 per element after G_t + u_{t-1} (the diagonal 1 + tau (d_x + d_y) comes
+// precombined per grid point in rdd), formed while the DST loads its tile.
+struct ResIn {
+  const double *G, *U;
+  const double *rxl, *rdd, *rxu, *ryl, *ryu;
+  int ny, nym, batch;
+  const int *mex;
+};
+
+// The DST of lengths 63, 127 and 255 over half of the odd extension (dst.cu), ncol = slabs nx
+// columns; RES: of the residual rin.  launch_dst_y picks it by dst2_fits.
+bool dst2_fits(int64_t ny, int64_t ncol, bool res_f32);
+template <typename Tin, typename Tout, typename T, bool RES>
+void launch_dst2(Ctx &c, const Tin *X, Tout *Y, int64_t ncol, int64_t ny, int64_t nx, const cpx<T> *tw, int mode,
+                 const int *skip, const ResIn &rin, const char *fam, double bytes);
 // Orthonormal DST-I along the middle axis of (nt, ny, nx); ny + 1 a power of two.
 // mode 0: store, 1: add into (double output only).
 template <typename Tin, typename Tout, typename T>
