@@ -15,7 +15,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OUT = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT, "libparadiag_gb300.so")
-SOURCES = ["fft.cu", "dst.cu", "pint.cu", "pint_chunk.cu", "krylov.cu", "krylov_members.cu", "control.cu", "plan.cu", "noalloc.cu", "batch.cu", "operator.cu"]
+SOURCES = ["fft.cu", "rfft_f32.cu", "rfft_f32i.cu", "rfft_f64.cu", "dst.cu", "pint.cu", "pint_chunk.cu", "krylov.cu", "krylov_members.cu", "control.cu", "plan.cu", "noalloc.cu", "batch.cu", "operator.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 
@@ -41,7 +41,7 @@ def _stale(target: str, deps) -> bool:
     return any(os.path.getmtime(d) > t for d in deps)
 
 
-def build(force: bool = False, verbose_ptxas: bool = False, jobs: int = 4) -> str:
+def build(force: bool = False, verbose_ptxas: bool = False, jobs: int = 8) -> str:
     os.makedirs(OUT, exist_ok=True)
     headers = [os.path.join(CSRC, h) for h in os.listdir(CSRC) if h.endswith((".h", ".cuh"))]
     headers.append(os.path.join(HERE, "..", "include", "paradiag.h"))

@@ -14,6 +14,7 @@
 
 #include "pd_control.cuh"
 #include "pd_fft.cuh"
+#include "pd_fft_tail.cuh"
 
 namespace pd {
 
@@ -125,40 +126,6 @@ __device__ void r2c_store(const cpx<T> *buf, int n, int logn, int64_t x0, int64_
       r = mk<T>(T(0.5) * (zk.y + zm.y), T(-0.5) * (zk.x - zm.x));
     }
     S[(int64_t)k * lds + col] = r;
-  }
-}
-
-// Sum of squares of the transformed data (per thread: ss), reduced over the launch: each
-// CTA stores its partial, and the last CTA to finish (no CTA waits for another) adds the
-// partials in a fixed order and stores the square root into *rn.dst.
-__device__ void rhs_norm_finish(float ss, const RhsNorm &rn) {
-  __shared__ double red[32];
-  __shared__ int last;
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = blockDim.x >> 5;
-  ss = warp_sum(ss);  // binary32 within a warp (a reference scale; FP64 adds cost GB300's FP64 pipe)
-  if (l == 0) red[w] = (double)ss;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int i = 0; i < nw; ++i) t += red[i];
-    rn.part[blockIdx.x] = t;
-    __threadfence();
-    last = atomicAdd(rn.counter, 1) == (int)gridDim.x - 1;
-  }
-  __syncthreads();
-  if (!last) return;
-  __threadfence();
-  double t = 0.0;
-  for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) t += __ldcg(rn.part + i);
-  t = warp_sum(t);
-  __syncthreads();  // red is reused
-  if (l == 0) red[w] = t;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double s2 = 0.0;
-    for (int i = 0; i < nw; ++i) s2 += red[i];
-    *rn.dst = sqrt(s2);
-    *rn.counter = 0;
   }
 }
 
@@ -431,8 +398,11 @@ __global__ void __launch_bounds__(256) k_fft_c2r(const cpx<T> *__restrict__ S, i
       for (int i = 0; i < 16; ++i) {
         const int idx = r + i * nb;
         const int kk = idx <= half ? idx : n - idx;
-        const cpx<T> A = ca < ncols ? S[(int64_t)kk * lds + ca] : mk<T>(T(0), T(0));
-        const cpx<T> B = cb < ncols ? S[(int64_t)kk * lds + cb] : mk<T>(T(0), T(0));
+        cpx<T> A = ca < ncols ? S[(int64_t)kk * lds + ca] : mk<T>(T(0), T(0));
+        cpx<T> B = cb < ncols ? S[(int64_t)kk * lds + cb] : mk<T>(T(0), T(0));
+        // rows 0 and n/2 are their own conjugates: an imaginary part there is not part of the real
+        // result (left in, it would reach the other column of the pair)
+        if (kk == 0 || kk == half) A.y = B.y = T(0);
         // conj(A + i B) at kk <= n/2; the conjugate half at n - kk
         z[i] = idx <= half ? mk<T>(A.x - B.y, -(A.y + B.x)) : mk<T>(A.x + B.y, A.y - B.x);
       }
@@ -466,6 +436,7 @@ __global__ void __launch_bounds__(256) k_fft_c2r(const cpx<T> *__restrict__ S, i
           const int kk = idx / np;
           const int p = idx - kk * np;
           cpx<T> *ser = buf + (size_t)p * series_stride(n);
+          if (kk == 0 || kk == half) A[u].y = B[u].y = T(0);  // (see the radix-16 branch)
           // conj(A + i B) = (A.x - B.y) - i (A.y + B.x); at n - kk the conjugate half
           // gives (A.x + B.y) + i (A.y - B.x)
           ser[bitrev(kk, logn)] = mk<T>(A[u].x - B[u].y, -(A[u].y + B[u].x));
@@ -517,57 +488,7 @@ __global__ void __launch_bounds__(256) k_fft_c2r(const cpx<T> *__restrict__ S, i
       ss = fmaf(vf, vf, ss);
     }
   }
-  if (colsum) {
-    // per-column sums of squares: blockDim.x is a multiple of TX, so every element a
-    // thread wrote lies in column threadIdx.x % TX
-    __shared__ double cred[256];
-    cred[threadIdx.x] = (double)ss;
-    __syncthreads();
-    if ((int)threadIdx.x < TX) {
-      double t = 0.0;
-      for (int i = threadIdx.x; i < (int)blockDim.x; i += TX) t += cred[i];
-      if (x0 + threadIdx.x < ncols) colsum[x0 + threadIdx.x] = t;
-    }
-  }
-  if (norm_part) {
-    const double sd = warp_sum((double)ss);
-    __shared__ double red[32];
-    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-    __syncthreads();
-    if (l == 0) red[w] = sd;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double t = 0.0;
-      for (int i = 0; i < (int)(blockDim.x >> 5); ++i) t += red[i];
-      norm_part[blockIdx.x] = t;
-    }
-    if (fin.enabled) {
-      // the last CTA to finish (no CTA waits) sums the squares and decides
-      __shared__ int last;
-      __threadfence();
-      __syncthreads();
-      if (threadIdx.x == 0) last = atomicAdd(fin.counter, 1) == (int)gridDim.x - 1;
-      __syncthreads();
-      if (last) {
-        __threadfence();
-        // every thread loads its share at once (the partials sit in L2, possibly on the
-        // other die: one round trip instead of one per partial), then a fixed-order sum
-        double t = 0.0;
-#pragma unroll 4
-        for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) t += norm_part[i];
-        t = warp_sum(t);
-        if (l == 0) red[w] = t;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-          t = 0.0;
-          for (int i = 0; i < (int)(blockDim.x >> 5); ++i) t += red[i];
-          fin.scal[S_D2] = t;
-          *fin.counter = 0;
-          refine_decide(fin.scal, fin.flags, fin.rc, fin.use_handle, fin.h);
-        }
-      }
-    }
-  }
+  c2r_finish<TX, 256>(ss, x0, ncols, colsum, norm_part, fin);
 }
 
 // Orthonormal DST-I along y via a length N = 2(ny+1) complex FFT of the odd
@@ -781,6 +702,9 @@ void launch_fft_r2c(Ctx &c, const Tin *X, int64_t ldx, int64_t ncols, int n, con
   const size_t smem = (size_t)(TX / 2) * fft_sst<T>(c, n) * sizeof(cpx<T>);
   const int grid = (int)((ncols + TX - 1) / TX);
   const double bytes = (double)n * ncols * sizeof(Tin) + (double)(n / 2 + 1) * ncols * sizeof(cpx<T>);
+  if (rfft_built<T>(c, n, ncols))
+    return rfft_launch<T, Tin>(c, X, ldx, ncols, n, tw, S, lds, rs, rn,
+                                      sizeof(T) == 8 ? "fft_r2c_f64" : "fft_r2c_f32", bytes);
   c.launch(sizeof(T) == 8 ? "fft_r2c_f64" : "fft_r2c_f32", bytes, [&] {
     PD_TX_DISPATCH(TX, {
       if (use_r16<T>(c, n)) {
@@ -832,6 +756,9 @@ void launch_fft_c2r(Ctx &c, const cpx<T> *S, int64_t lds, int64_t ncols, int n, 
   if (nparts) *nparts = grid;
   const double obytes = (mode == 2) ? 4.0 : (mode == 1 ? 16.0 : 8.0);
   const double bytes = (double)(n / 2 + 1) * ncols * sizeof(cpx<T>) + (double)n * ncols * obytes;
+  if (rfft_built<T>(c, n, ncols))
+    return crfft_launch<T>(c, S, lds, ncols, n, tw, out, ldo, mode, norm_part, nparts, fin, rsi, colsum, mex, mnx, skip,
+                           sizeof(T) == 8 ? "fft_c2r_f64" : "fft_c2r_f32", bytes);
   c.launch(sizeof(T) == 8 ? "fft_c2r_f64" : "fft_c2r_f32", bytes, [&] {
     PD_TX_DISPATCH(TX, {
       if (use_r16<T>(c, n)) {

@@ -102,10 +102,76 @@ __device__ __forceinline__ void dft32(cpx<T> (&x)[32]) {
     x[k + 16] = sub(e[k], t);
   }
 }
+// exp(-2 pi i m / N), 0 <= m <= N / 4, N a power of two up to 64
+template <typename T, int N>
+__device__ __forceinline__ cpx<T> wn(int m) {
+  constexpr double c[17] = {1.0, 0.9951847266721968862448, 0.9807852804032304491261, 0.9569403357322088649357,
+                            0.9238795325112867561281, 0.8819212643483550297127, 0.8314696123025452370787,
+                            0.7730104533627369608109, 0.7071067811865475244008, 0.6343932841636454982151,
+                            0.5555702330196022247428, 0.4713967368259976485563, 0.3826834323650897717284,
+                            0.2902846772544623676361, 0.1950903220161282678482, 0.0980171403295606019941, 0.0};
+  const int t = m * (64 / N);  // c[k] = cos(pi k / 32)
+  return mk<T>((T)c[t], (T)-c[16 - t]);
+}
+
+// Real input: X[k] = sum_i x[O + S i] w^{ik}, w = exp(-2 pi i / N), k = 0 .. N/2 (X[0] and X[N/2] real),
+// by halving: even and odd samples, X[k] = E[k] + w^k O[k], X[N/2 - k] = conj(E[k] - w^k O[k]).
+template <typename T, int N, int S, int O, int M>
+__device__ __forceinline__ void rdft(const T (&x)[M], cpx<T> (&X)[N / 2 + 1]) {
+  if constexpr (N == 4) {
+    const T a = x[O] + x[O + 2 * S], b = x[O + S] + x[O + 3 * S];
+    X[0] = mk<T>(a + b, T(0));
+    X[1] = mk<T>(x[O] - x[O + 2 * S], x[O + 3 * S] - x[O + S]);
+    X[2] = mk<T>(a - b, T(0));
+  } else {
+    cpx<T> e[N / 4 + 1], o[N / 4 + 1];
+    rdft<T, N / 2, 2 * S, O, M>(x, e);
+    rdft<T, N / 2, 2 * S, O + S, M>(x, o);
+    X[0] = mk<T>(e[0].x + o[0].x, T(0));
+    X[N / 2] = mk<T>(e[0].x - o[0].x, T(0));
+    X[N / 4] = mk<T>(e[N / 4].x, -o[N / 4].x);
+#pragma unroll
+    for (int k = 1; k < N / 4; ++k) {
+      const cpx<T> t = mul(wn<T, N>(k), o[k]);
+      X[k] = add(e[k], t);
+      X[N / 2 - k] = conjg(sub(e[k], t));
+    }
+  }
+}
+
+// Hermitian input (X[N - k] = conj X[k], given k = 0 .. N/2; the imaginary parts of X[0] and X[N/2] do
+// not count), real output x[O + S i] = sum_k X[k] w^{ik}: the transpose of rdft.
+template <typename T, int N, int S, int O, int M>
+__device__ __forceinline__ void hdft(const cpx<T> (&X)[N / 2 + 1], T (&x)[M]) {
+  if constexpr (N == 4) {
+    const T s = X[0].x + X[2].x, d = X[0].x - X[2].x, p = X[1].x + X[1].x, q = X[1].y + X[1].y;
+    x[O] = s + p;
+    x[O + 2 * S] = s - p;
+    x[O + S] = d + q;
+    x[O + 3 * S] = d - q;
+  } else {
+    cpx<T> a[N / 4 + 1], b[N / 4 + 1];
+    a[0] = mk<T>(X[0].x + X[N / 2].x, T(0));
+    b[0] = mk<T>(X[0].x - X[N / 2].x, T(0));
+    a[N / 4] = mk<T>(X[N / 4].x + X[N / 4].x, T(0));
+    b[N / 4] = mk<T>(X[N / 4].y + X[N / 4].y, T(0));
+#pragma unroll
+    for (int k = 1; k < N / 4; ++k) {
+      const cpx<T> v = conjg(X[N / 2 - k]);
+      a[k] = add(X[k], v);
+      b[k] = mul(wn<T, N>(k), sub(X[k], v));
+    }
+    hdft<T, N / 2, 2 * S, O, M>(a, x);
+    hdft<T, N / 2, 2 * S, O + S, M>(b, x);
+  }
+}
+
 template <typename T, int R>
 __device__ __forceinline__ void dft_reg(cpx<T> (&x)[R]) {
-  static_assert(R == 8 || R == 16 || R == 32, "built sizes");
-  if constexpr (R == 8)
+  static_assert(R == 4 || R == 8 || R == 16 || R == 32, "built sizes");
+  if constexpr (R == 4)
+    radix4_fwd(x[0], x[1], x[2], x[3]);
+  else if constexpr (R == 8)
     dft8(x);
   else if constexpr (R == 16)
     dft16(x);

@@ -187,6 +187,23 @@ struct StepFinish {
   int use_handle;
   cudaGraphConditionalHandle h;
 };
+// The same transforms in two register passes (rfft.cuh), for n = 32 .. 2048; the launchers above
+// and below pick them unless the caller chose a first-stage radix or a tile width.
+// binary64 transforms of 512 points and more with too few columns for the wide tiles stay in
+// fft.cu: 511 columns of 512 points 24 / 29 us here against 22 / 25 us (forward / inverse), 1023
+// columns of 1024 points 60 / 70 us against 65 / 66 us.
+template <typename T>
+bool rfft_built(const Ctx &c, int n, int64_t ncols) {
+  if (c.fft_radix != 0 || c.fft_cols != 0 || n < 32 || n > 2048) return false;
+  return sizeof(T) == 4 || n <= 256 || ncols * n >= (int64_t)16384 * sm_count();
+}
+template <typename T, typename Tin>
+void rfft_launch(Ctx &c, const Tin *X, int64_t ldx, int64_t ncols, int n, const cpx<T> *tw, cpx<T> *S, int64_t lds,
+                 const T *rs, const RhsNorm &rn, const char *fam, double bytes);
+template <typename T>
+void crfft_launch(Ctx &c, const cpx<T> *S, int64_t lds, int64_t ncols, int n, const cpx<T> *tw, void *out, int64_t ldo,
+                  int mode, double *norm_part, int *nparts, const StepFinish &fin, const T *rsi, double *colsum,
+                  const int *mex, int mnx, const int *skip, const char *fam, double bytes);
 // Inverse DFT along time of a half spectrum; mode 0: store double, 1: add into
 // double, 2: store float.  norm_part (may be null) receives per-CTA sums of the
 // squared output values; *nparts = number of CTAs.  colsum (may be null) receives
