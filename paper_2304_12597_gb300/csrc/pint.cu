@@ -975,7 +975,7 @@ void launch_zsum(Ctx &c, int nf, int64_t n, const cpx<T> *H, int64_t ldh, const 
                  skip_flag, tail, mlen, h0);
     } else {
       const int grid = (int)((n + 7) / 8);
-      if (smem > 48 * 1024)
+      if (smem > 24 * 1024)  // beside the tail's static arrays, 32 KB already need the opt-in
         allow_dyn_smem((const void *)k_zsum<T, 8, 64>);
       pdl_launch(c.pdl, k_zsum<T, 8, 64>, dim3(grid), dim3(512), smem, c.stream, nf, n, H, ldh, omega, z,
                  skip_flag, tail, mlen, h0);
