@@ -1,9 +1,10 @@
 // Per-problem scaling for batched plans: `batch` independent problems share one
 // plan as a block-diagonal problem (slot b = columns [b*nxm, (b+1)*nxm) of every
 // time row).  The Krylov and refinement stopping rules measure the whole stack, so
-// every problem is first scaled to unit Frobenius norm (up to a factor of two) and
-// scaled back after the solve.  The scale factors are powers of two: the scaling is
-// exact and costs integer work on the exponent field, not FP64 multiplies.
+// every problem is solved scaled to unit Frobenius norm (up to a factor of two).  The
+// scale factors are powers of two, found here; the transforms apply them on load and
+// undo them on store (SlotScale), by integer work on the exponent field.  (As passes of
+// their own, scaling G and unscaling U took 184 of 2913 us on 32 x heat1d_1023x1024.)
 #include <algorithm>
 
 #include "pd_internal.h"
@@ -37,9 +38,10 @@ __global__ void __launch_bounds__(256) k_batch_sumsq(const double *__restrict__ 
 // values the paired real DFTs leave in its columns, and it takes no part in the
 // refinement decision.
 __global__ void k_batch_exponents(int batch, int nc, const double *__restrict__ part, int *__restrict__ ex,
-                                  int *__restrict__ zero) {
+                                  int *__restrict__ zero, const double *G, const double **gslot) {
   grid_dep_wait();
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
+  if (b == 0) *gslot = G;
   if (b >= batch) return;
   double s = 0.0;
   for (int c = 0; c < nc; ++c) s += part[(int64_t)b * nc + c];
@@ -53,42 +55,24 @@ __global__ void k_batch_exponents(int batch, int nc, const double *__restrict__ 
   zero[b] = s == 0.0 ? 1 : 0;
 }
 
-// Y = X * 2^(sign * ex[slot]) over the (nt, ld) array, one time row per blockIdx.y;
-// Y may alias X.  With nxb != NULL, columns past problem b's n_x, and every column of an
-// all-zero problem (zero[b]), are set to zero (they are decoupled from the problem, but
-// the paired real-to-complex DFT leaves rounding-level values there).
-__global__ void __launch_bounds__(256) k_batch_scale(const double *X, double *Y, int ld, int nxm,
-                                                     const int *__restrict__ ex, int sign,
-                                                     const int *__restrict__ nxb, const int *__restrict__ zero) {
-  grid_dep_wait();
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= ld) return;
-  const int b = j / nxm;
-  const int64_t i = (int64_t)blockIdx.y * ld + j;
-  Y[i] = (nxb && (j - b * nxm >= nxb[b] || zero[b])) ? 0.0 : pow2_scale(X[i], sign * ex[b]);
-}
-
-void launch_batch_normalize(Ctx &c, const double *G, double *Gs, int64_t nt, int batch, int nxm, int nc,
-                            double *part, int *ex, int *zero) {
+void launch_batch_exponents(Ctx &c, const double *G, int64_t nt, int batch, int nxm, int nc, double *part, int *ex,
+                            int *zero, const double **gslot) {
   const int64_t ld = (int64_t)batch * nxm;
   c.launch("batch_scale", (double)nt * ld * 8.0, [&] {
     pdl_launch(c.pdl, k_batch_sumsq, dim3(nc, batch), dim3(256), 0, c.stream, G, nt, ld, nxm, nc, part);
   });
-  c.launch("batch_scale", 0.0, [&] { pdl_launch(c.pdl, k_batch_exponents, dim3((batch + 127) / 128), dim3(128), 0, c.stream, batch, nc, part, ex,
-                                                        zero); });
-  const dim3 grid((unsigned)((ld + 255) / 256), (unsigned)nt);
-  c.launch("batch_scale", (double)nt * ld * 16.0,
-           [&] { pdl_launch(c.pdl, k_batch_scale, grid, dim3(256), 0, c.stream, G, Gs, (int)ld, nxm, (const int *)ex, 1,
-                                  (const int *)nullptr, (const int *)nullptr); });
+  c.launch("batch_scale", 0.0, [&] {
+    pdl_launch(c.pdl, k_batch_exponents, dim3((batch + 127) / 128), dim3(128), 0, c.stream, batch, nc, part, ex, zero, G,
+               gslot);
+  });
 }
 
 // A problem joining a running batch (join[b]): its U slot starts at zero and its refinement
 // state restarts; so does every unused slot (zero[b]: an all-zero right-hand side, whose U
-// may hold anything); the other slots' U goes back into the solve's units, U * 2^ex[b]
-// (exact).
-__global__ void __launch_bounds__(256) k_member_join(double *U, int ld, int nxm, int batch, const int *__restrict__ ex,
-                                                     const int *__restrict__ join, const int *__restrict__ zero,
-                                                     int *msw, double *prev, double *ref2, int *mex, int *mconv) {
+// may hold anything).  The other slots are not touched.
+__global__ void __launch_bounds__(256) k_member_join(double *U, int ld, int nxm, int batch, const int *__restrict__ join,
+                                                     const int *__restrict__ zero, int *msw, double *prev, double *ref2,
+                                                     int *mex, int *mconv) {
   grid_dep_wait();
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (blockIdx.y == 0 && j < batch && (join[j] || zero[j])) {  // (an unused slot's mex may be stale)
@@ -100,27 +84,17 @@ __global__ void __launch_bounds__(256) k_member_join(double *U, int ld, int nxm,
   }
   if (j >= ld) return;
   const int b = j / nxm;
-  const int64_t i = (int64_t)blockIdx.y * ld + j;
-  U[i] = (join[b] || zero[b]) ? 0.0 : pow2_scale(U[i], ex[b]);
+  if (join[b] || zero[b]) U[(int64_t)blockIdx.y * ld + j] = 0.0;
 }
 
-void launch_member_join(Ctx &c, double *U, int64_t nt, int batch, int nxm, const int *ex, const int *join,
-                        const int *zero, int *msw, double *prev, double *ref2, int *mex, int *mconv) {
+void launch_member_join(Ctx &c, double *U, int64_t nt, int batch, int nxm, const int *join, const int *zero, int *msw,
+                        double *prev, double *ref2, int *mex, int *mconv) {
   const int64_t ld = (int64_t)batch * nxm;
   const dim3 grid((unsigned)((std::max<int64_t>(ld, batch) + 255) / 256), (unsigned)nt);
-  c.launch("batch_scale", (double)nt * ld * 16.0, [&] {
-    pdl_launch(c.pdl, k_member_join, grid, dim3(256), 0, c.stream, U, (int)ld, nxm, batch, ex, join, zero, msw, prev,
-               ref2, mex, mconv);
+  c.launch("batch_join", (double)nt * ld * 8.0, [&] {
+    pdl_launch(c.pdl, k_member_join, grid, dim3(256), 0, c.stream, U, (int)ld, nxm, batch, join, zero, msw, prev, ref2,
+               mex, mconv);
   });
-}
-
-void launch_batch_unscale(Ctx &c, double *U, int64_t nt, int batch, int nxm, const int *ex, const int *nxb,
-                          const int *zero) {
-  const int64_t ld = (int64_t)batch * nxm;
-  const dim3 grid((unsigned)((ld + 255) / 256), (unsigned)nt);
-  c.launch("batch_scale", (double)nt * ld * 16.0,
-           [&] { pdl_launch(c.pdl, k_batch_scale, grid, dim3(256), 0, c.stream, (const double *)U, U, (int)ld, nxm, ex, -1,
-                                  nxb, zero); });
 }
 
 // out[t][j] = in[t][j] * s[j] (in place allowed): the diagonal mass matrix's symmetric

@@ -35,6 +35,8 @@ namespace {
 struct Col {  // one column of a lane
   int64_t base;  // its first element (row 0) in the (slab, y, x) array
   bool in;
+  int ein, eout;  // batches: the problem's exact scaling, on binary64 input and off binary64 output
+  bool dead;      // the output of an all-zero problem: exact zeros
   // residual input: problem b, x, whether its slab is the first time, the x-coefficients
   int b, x;
   bool t0;
@@ -44,16 +46,23 @@ struct Col {  // one column of a lane
 }  // namespace
 
 // MODE 0: Y = DST X; 1: Y += DST X.  RES: the input is the FP64 residual of ResIn instead of X.
-template <typename Tin, typename Tout, typename T, int R1, int R2, int NW, int MINB, int MODE, bool RES>
+template <typename Tin, typename Tout, typename T, int R1, int R2, int NW, int MINB, int MODE, bool RES, bool SLOT>
 __global__ void __launch_bounds__(NW * 32, MINB)
     k_dst2(const Tin *__restrict__ X, Tout *__restrict__ Y, int64_t ncol, int64_t nx, const cpx<T> *__restrict__ tw,
-           T scale, const int *skip, ResIn rin) {
+           T scale, const int *skip, ResIn rin, SlotScale sc) {
   grid_dep_wait();
   if (skip && *skip) return;  // U already holds the result (Algorithm 3's U_1 exit)
   constexpr int N = R1 * R2 / 2, NY = N - 1, S = R1 + 1;
   extern __shared__ __align__(16) unsigned char smraw[];
   cpx<T> *sm = reinterpret_cast<cpx<T> *>(smraw);  // T_r[k1] at ((r S + k1) 32 + lane), T_r[-k1] at k1 -> R1 - k1, T_r[-R1/2] at R1
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if constexpr (SLOT) {
+    if constexpr (RES) {
+      rin.G = global_ptr(sc.G);
+    } else if constexpr (sizeof(Tin) == 8) {
+      if (sc.G) X = global_ptr(sc.G);
+    }
+  }
   Col c[2];
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
@@ -62,6 +71,15 @@ __global__ void __launch_bounds__(NW * 32, MINB)
     const int64_t slab = c[h].in ? g / nx : 0;
     const int x = c[h].in ? (int)(g - slab * nx) : 0;
     c[h].base = slab * (NY * nx) + x;
+    c[h].ein = c[h].eout = 0;
+    c[h].dead = false;
+    if constexpr (SLOT) {  // (with sc.G: a transform of the caller's G or of the residual; else one into U)
+      const int b = (int)(slab % sc.batch);
+      if (sc.G)
+        c[h].ein = sc.ex[b];
+      else
+        c[h].eout = -sc.ex[b], c[h].dead = sc.zero[b] != 0;
+    }
     if constexpr (RES) {
       // slabs are (time, problem) with the problems of a time row adjacent, as the rows of the
       // stacked grid are: G and U take the slab's own element index
@@ -103,7 +121,10 @@ __global__ void __launch_bounds__(NW * 32, MINB)
       r = fma(-q.cu, ur[u], r);
       r = fma(-rin.ryl[iy], ud[u], r);
       r = fma(-rin.ryu[iy], uu[u], r);
-      v[u] = cvt<T>(rin.mex ? pow2_scale(r, rin.mex[q.b]) : r);
+      if constexpr (SLOT)
+        v[u] = slot_load<T>(r, q.ein + rin.mex[q.b]);
+      else
+        v[u] = cvt<T>(r);
     }
   };
 
@@ -154,7 +175,14 @@ __global__ void __launch_bounds__(NW * 32, MINB)
       }
 #pragma unroll
       for (int i = 0; i < R1; ++i) {
-        const T a = cvt<T>(va[i]), b = cvt<T>(vb[i]);
+        T a, b;
+        if constexpr (SLOT && sizeof(Tin) == 8) {
+          a = slot_load<T>(va[i], c[0].ein);
+          b = slot_load<T>(vb[i], c[1].ein);
+        } else {
+          a = cvt<T>(va[i]);
+          b = cvt<T>(vb[i]);
+        }
         z[i] = i < R1 / 2 ? mk<T>(a, b) : mk<T>(-a, -b);
       }
     }
@@ -208,8 +236,20 @@ __global__ void __launch_bounds__(NW * 32, MINB)
         const int row = upper ? 2 * N - k - 1 : k - 1;
         const cpx<T> v = z[q0 + u];
         const T a = (upper ? -sa : sa) * v.y, b = (upper ? -sb : sb) * v.x;
-        if (row >= 0 && c[0].in) Y[c[0].base + (int64_t)row * nx] = MODE == 1 ? oa[u] + cvt<Tout>(a) : cvt<Tout>(a);
-        if (row >= 0 && c[1].in) Y[c[1].base + (int64_t)row * nx] = MODE == 1 ? ob[u] + cvt<Tout>(b) : cvt<Tout>(b);
+        Tout da, db;
+        if constexpr (SLOT && sizeof(Tout) == 8) {
+          da = slot_store(a, c[0].eout);
+          db = slot_store(b, c[1].eout);
+        } else {
+          da = cvt<Tout>(a);
+          db = cvt<Tout>(b);
+        }
+        if (MODE == 1) {
+          da = oa[u] + da;
+          db = ob[u] + db;
+        }
+        if (row >= 0 && c[0].in) Y[c[0].base + (int64_t)row * nx] = SLOT && c[0].dead ? Tout(0) : da;
+        if (row >= 0 && c[1].in) Y[c[1].base + (int64_t)row * nx] = SLOT && c[1].dead ? Tout(0) : db;
       }
     }
   }
@@ -225,17 +265,25 @@ bool dst2_fits(int64_t ny, int64_t ncol, bool res_f32) {
 
 template <typename Tin, typename Tout, typename T, int R1, int R2, int NW, int MINB, bool RES>
 static void launch_size(Ctx &c, const Tin *X, Tout *Y, int64_t ncol, int64_t ny, int64_t nx, const cpx<T> *tw, int mode,
-                        const int *skip, const ResIn &rin, const char *fam, double bytes) {
+                        const int *skip, const ResIn &rin, const SlotScale &sc, const char *fam, double bytes) {
   const size_t smem = (size_t)(R2 / 2 + 1) * (R1 + 1) * 32 * sizeof(cpx<T>);
   const T scale = (T)sqrt(2.0 / (double)(ny + 1));
   const unsigned grid = (unsigned)((ncol + 63) / 64);
-  auto kern = k_dst2<Tin, Tout, T, R1, R2, NW, MINB, 0, RES>;
+  auto kern = k_dst2<Tin, Tout, T, R1, R2, NW, MINB, 0, RES, false>;
   if constexpr (!RES && sizeof(Tout) == 8) {
-    if (mode) kern = k_dst2<Tin, Tout, T, R1, R2, NW, MINB, 1, RES>;
+    if (mode) kern = k_dst2<Tin, Tout, T, R1, R2, NW, MINB, 1, RES, false>;
+  }
+  if constexpr (R1 * R2 < 512) {  // (batches of n_y = 255, n_x <= 32 stay with k_dst_y)
+    if (sc.ex) {
+      kern = k_dst2<Tin, Tout, T, R1, R2, NW, MINB, 0, RES, true>;
+      if constexpr (!RES && sizeof(Tout) == 8) {
+        if (mode) kern = k_dst2<Tin, Tout, T, R1, R2, NW, MINB, 1, RES, true>;
+      }
+    }
   }
   c.launch(fam, bytes, [&] {
     if (smem > 48 * 1024) allow_dyn_smem((const void *)kern);
-    pdl_launch(c.pdl, kern, dim3(grid), dim3(NW * 32), smem, c.stream, X, Y, ncol, nx, tw, scale, skip, rin);
+    pdl_launch(c.pdl, kern, dim3(grid), dim3(NW * 32), smem, c.stream, X, Y, ncol, nx, tw, scale, skip, rin, sc);
   });
 }
 
@@ -244,19 +292,19 @@ static void launch_size(Ctx &c, const Tin *X, Tout *Y, int64_t ncol, int64_t ny,
 // warps with 2 to 4 CTAs per SM: 255 59 us against 75 and 78, the others within 5 %.
 template <typename Tin, typename Tout, typename T, bool RES>
 void launch_dst2(Ctx &c, const Tin *X, Tout *Y, int64_t ncol, int64_t ny, int64_t nx, const cpx<T> *tw, int mode,
-                 const int *skip, const ResIn &rin, const char *fam, double bytes) {
+                 const int *skip, const ResIn &rin, const SlotScale &sc, const char *fam, double bytes) {
   constexpr int B = sizeof(T) == 8 ? 1 : 2;
   if (ny == 63)
-    launch_size<Tin, Tout, T, 16, 8, 5, sizeof(T) == 8 ? 2 : 4, RES>(c, X, Y, ncol, ny, nx, tw, mode, skip, rin, fam, bytes);
+    launch_size<Tin, Tout, T, 16, 8, 5, sizeof(T) == 8 ? 2 : 4, RES>(c, X, Y, ncol, ny, nx, tw, mode, skip, rin, sc, fam, bytes);
   else if (ny == 255)
-    launch_size<Tin, Tout, T, 16, 32, 9, B, RES>(c, X, Y, ncol, ny, nx, tw, mode, skip, rin, fam, bytes);
+    launch_size<Tin, Tout, T, 16, 32, 9, B, RES>(c, X, Y, ncol, ny, nx, tw, mode, skip, rin, sc, fam, bytes);
   else if constexpr (!(RES && sizeof(T) == 4))
-    launch_size<Tin, Tout, T, 16, 16, 9, B, RES>(c, X, Y, ncol, ny, nx, tw, mode, skip, rin, fam, bytes);
+    launch_size<Tin, Tout, T, 16, 16, 9, B, RES>(c, X, Y, ncol, ny, nx, tw, mode, skip, rin, sc, fam, bytes);
 }
 
 #define PD_DST2(TIN, TOUT, T, RES)                                                                                   \
   template void launch_dst2<TIN, TOUT, T, RES>(Ctx &, const TIN *, TOUT *, int64_t, int64_t, int64_t, const cpx<T> *, \
-                                               int, const int *, const ResIn &, const char *, double);
+                                               int, const int *, const ResIn &, const SlotScale &, const char *, double);
 PD_DST2(double, float, float, false)
 PD_DST2(float, float, float, false)
 PD_DST2(float, double, float, false)

@@ -222,14 +222,24 @@ __device__ void r2c_store16(const cpx<T> *buf, int n, int64_t x0, int64_t ncols,
   }
 }
 
+// an input sample of a transform: binary64 with its problem's scaling, or as it is
+template <bool SLOT, typename T, typename Tin>
+__device__ __forceinline__ T in_load(Tin x, int ex) {
+  if constexpr (SLOT && sizeof(Tin) == 8)
+    return slot_load<T>(x, ex);
+  else
+    return cvt<T>(x);
+}
+
 // Forward DFT of TX columns per CTA (n >= 16): each thread takes a (column pair, block)
 // item: loads the block's 16 time samples of both columns (packed z = a + i b), dft16,
 // writes the block; then the later stages and the separated half spectra.
-template <typename T, typename Tin, int TX>
+template <typename T, typename Tin, int TX, bool SLOT>
 __global__ void __launch_bounds__(sizeof(T) == 8 ? 256 : 512)
     k_fft_r2c16(const Tin *__restrict__ X, int64_t ldx, int64_t ncols, int n, int logn, const cpx<T> *__restrict__ tw,
-                cpx<T> *__restrict__ S, int64_t lds, const T *__restrict__ rs, RhsNorm rn) {
+                cpx<T> *__restrict__ S, int64_t lds, const T *__restrict__ rs, RhsNorm rn, SlotScale sc) {
   grid_dep_wait();
+  if constexpr (SLOT && sizeof(Tin) == 8) X = global_ptr(sc.G);
   extern __shared__ __align__(16) unsigned char smraw[];
   cpx<T> *buf = reinterpret_cast<cpx<T> *>(smraw);
   constexpr int NP = TX / 2;
@@ -241,12 +251,13 @@ __global__ void __launch_bounds__(sizeof(T) == 8 ? 256 : 512)
     const int r = bitrev(g, lb);
     const int64_t ca = x0 + 2 * p, cb = ca + 1;
     const bool va = ca < ncols, vb = cb < ncols;
+    const int ea = SLOT && va ? sc.ex[ca / sc.mnx] : 0, eb = SLOT && vb ? sc.ex[cb / sc.mnx] : 0;
     cpx<T> z[16];
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
       const int64_t j = r + i * nb;
       const Tin *row = X + j * ldx;
-      z[i] = mk<T>(va ? cvt<T>(row[ca]) : T(0), vb ? cvt<T>(row[cb]) : T(0));
+      z[i] = mk<T>(va ? in_load<SLOT, T>(row[ca], ea) : T(0), vb ? in_load<SLOT, T>(row[cb], eb) : T(0));
     }
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
@@ -264,12 +275,13 @@ __global__ void __launch_bounds__(sizeof(T) == 8 ? 256 : 512)
   if (rn.part) rhs_norm_finish((float)ss, rn);
 }
 
-template <typename T, typename Tin, int TX>
+template <typename T, typename Tin, int TX, bool SLOT>
 __global__ void __launch_bounds__(kFftMaxThreads) k_fft_r2c(const Tin *__restrict__ X, int64_t ldx, int64_t ncols,
                                                  int n, int logn, const cpx<T> *__restrict__ tw,
                                                  cpx<T> *__restrict__ S, int64_t lds, const T *__restrict__ rs,
-                                                 RhsNorm rn) {
+                                                 RhsNorm rn, SlotScale sc) {
   grid_dep_wait();
+  if constexpr (SLOT && sizeof(Tin) == 8) X = global_ptr(sc.G);
   extern __shared__ __align__(16) unsigned char smraw[];
   cpx<T> *buf = reinterpret_cast<cpx<T> *>(smraw);
   const int64_t x0 = (int64_t)blockIdx.x * TX;
@@ -286,7 +298,7 @@ __global__ void __launch_bounds__(kFftMaxThreads) k_fft_r2c(const Tin *__restric
       const int sl = idx / TX;
       const int j = idx < total ? bitrev(sl, logn) : 0;
       const int64_t col = x0 + (idx - sl * TX);
-      v[u] = (idx < total && col < ncols) ? cvt<T>(X[(int64_t)j * ldx + col]) : T(0);
+      v[u] = (idx < total && col < ncols) ? in_load<SLOT, T>(X[(int64_t)j * ldx + col], SLOT ? sc.ex[col / sc.mnx] : 0) : T(0);
     }
 #pragma unroll
     for (int u = 0; u < kLoadBatch; ++u) {
@@ -309,15 +321,16 @@ __global__ void __launch_bounds__(kFftMaxThreads) k_fft_r2c(const Tin *__restric
 // Same transform of the 1D FP64 residual r = G_t + u_{t-1} - (I + tau K) u_t, formed
 // while the tile is loaded (rx = (tau lo, 1 + tau diag, tau up)); neighbour columns
 // outside the tile come from L1/L2.
-template <typename T, int TX>
+template <typename T, int TX, bool SLOT>
 __global__ void __launch_bounds__(kFftMaxThreads, 2) k_fft_r2c_res(const double *__restrict__ G, const double *__restrict__ U,
                                                      int64_t ncols, int n, int logn, const double *__restrict__ rxl,
                                                      const double *__restrict__ rxd,
                                                      const double *__restrict__ rxu,
                                                      const cpx<T> *__restrict__ tw, cpx<T> *__restrict__ S,
                                                      int64_t lds, const T *__restrict__ rs,
-                                                     const int *__restrict__ mex, int mnx, RhsNorm rn) {
+                                                     const int *__restrict__ mex, int mnx, RhsNorm rn, SlotScale sc) {
   grid_dep_wait();
+  if constexpr (SLOT) G = global_ptr(sc.G);
   extern __shared__ __align__(16) unsigned char smraw[];
   cpx<T> *buf = reinterpret_cast<cpx<T> *>(smraw);
   const int64_t x0 = (int64_t)blockIdx.x * TX;
@@ -331,8 +344,8 @@ __global__ void __launch_bounds__(kFftMaxThreads, 2) k_fft_r2c_res(const double 
   const double cd = live ? rxd[col] : 0.0;
   const double cu = (live && col + 1 < ncols) ? rxu[col] : 0.0;
   const int64_t ol = col > 0 ? -1 : 0, ou = col + 1 < ncols ? 1 : 0;  // in-range neighbour offsets
-  // batched plans: problem (col / mnx) scaled by 2^mex[problem] (exact)
-  const T msc = (mex && live) ? (T)ldexp(1.0, mex[col / mnx]) : T(1);
+  // batched plans: problem (col / mnx) scaled by 2^(ex + mex) (exact)
+  const int ex = SLOT && live ? mex[col / mnx] + sc.ex[col / mnx] : 0;
   T *col_buf = reinterpret_cast<T *>(buf + (size_t)(c >> 1) * series_stride(n)) + (c & 1);
   constexpr int kB = kLoadBatch / 2;  // five FP64 loads per element
   T ss = T(0);  // squares of the residual (rn)
@@ -359,7 +372,7 @@ __global__ void __launch_bounds__(kFftMaxThreads, 2) k_fft_r2c_res(const double 
         const int j = bitrev(sq, logn);
         // four FP64 operations per element (GB300 runs FP64 at ~1/64 of the FP32 rate)
         const double res = fma(-cu, ur[q], fma(-cl, ul[q], fma(-cd, uc[q], g[q] + um[q])));
-        const T r = cvt<T>(res) * msc;
+        const T r = SLOT ? slot_load<T>(res, ex) : cvt<T>(res);
         col_buf[2 * sq] = rs ? r * rs[j] : r;
         ss += r * r;
       }
@@ -373,13 +386,14 @@ __global__ void __launch_bounds__(kFftMaxThreads, 2) k_fft_r2c_res(const double 
 
 // Inverse: Z[k] = A[k] + i B[k] over the full spectrum (A[n-k] = conj A[k]);
 // z = IDFT(Z) = conj(DFT(conj Z)) / n; column 2p = Re z, column 2p+1 = Im z.
-template <typename T, int TX, bool R16>
+template <typename T, int TX, bool R16, bool SLOT>
 __global__ void __launch_bounds__(256) k_fft_c2r(const cpx<T> *__restrict__ S, int64_t lds, int64_t ncols,
                                                  int n, int logn, const cpx<T> *__restrict__ tw,
                                                  void *__restrict__ out, int64_t ldo, int mode,
                                                  double *__restrict__ norm_part, StepFinish fin,
                                                  const T *__restrict__ rsi, double *__restrict__ colsum,
-                                                 const int *__restrict__ mex, int mnx, const int *skip) {
+                                                 const int *__restrict__ mex, int mnx, const int *skip,
+                                                 SlotScale slot) {
   grid_dep_wait();
   if (skip && *skip) return;  // U already holds the result (Algorithm 3's U_1 exit)
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -453,6 +467,16 @@ __global__ void __launch_bounds__(256) k_fft_c2r(const cpx<T> *__restrict__ S, i
     const int64_t c0 = x0 + (int64_t)(threadIdx.x % TX);
     if (c0 < ncols) inv_n = (T)ldexp((double)inv_n, -mex[c0 / mnx]);
   }
+  int ex = 0;
+  bool dead = false;  // (see k_crfft)
+  if constexpr (SLOT) {
+    const int64_t c0 = x0 + (int64_t)(threadIdx.x % TX);
+    if (mode != 2 && c0 < ncols) {
+      const int b = (int)(c0 / slot.mnx);
+      ex = -slot.ex[b];
+      dead = slot.zero[b] || c0 - (int64_t)b * slot.mnx >= slot.nxb[b];
+    }
+  }
   float ss = 0.0f;  // a few dozen squares per thread; the stop rule needs a few digits
   const int tot2 = n * TX;
   for (int i0 = threadIdx.x; i0 < tot2; i0 += kEpiBatch * blockDim.x) {
@@ -477,12 +501,16 @@ __global__ void __launch_bounds__(256) k_fft_c2r(const cpx<T> *__restrict__ S, i
       const T sc = rsi ? inv_n * rsi[j] : inv_n;
       const T v = ((c & 1) == 0) ? r.x * sc : -r.y * sc;
       const int64_t o = (int64_t)j * ldo + col;
-      if (mode == 0) {
-        reinterpret_cast<double *>(out)[o] = cvt<double>(v);
-      } else if (mode == 1) {
-        reinterpret_cast<double *>(out)[o] = old[u] + cvt<double>(v);
-      } else {
+      if (mode == 2) {
         reinterpret_cast<float *>(out)[o] = (float)v;
+      } else {
+        double d;
+        if constexpr (SLOT)
+          d = slot_store(v, ex);
+        else
+          d = cvt<double>(v);
+        if (mode == 1) d = old[u] + d;
+        reinterpret_cast<double *>(out)[o] = SLOT && dead ? 0.0 : d;
       }
       const float vf = (float)v;
       ss = fmaf(vf, vf, ss);
@@ -502,7 +530,7 @@ template <typename Tin, typename Tout, typename T, int TX, bool R16, bool RES>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 5 : 1) k_dst_y(const Tin *__restrict__ X, Tout *__restrict__ Y, int64_t ny,
                                                int64_t nx, int N, int logN,
                                                const cpx<T> *__restrict__ tw, T scale, int mode, const int *skip,
-                                               ResIn rin, size_t res_off) {
+                                               ResIn rin, size_t res_off, SlotScale sc) {
   grid_dep_wait();
   if (skip && *skip) return;  // U already holds the result (Algorithm 3's U_1 exit)
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -510,6 +538,15 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 5 : 1) k_dst_y(const Tin
   const int ntile = (int)((nx + TX - 1) / TX);
   const int64_t t = blockIdx.x / ntile;
   const int64_t x0 = (int64_t)(blockIdx.x % ntile) * TX;
+  // batches: with sc.G the problem's scaling goes onto the input (the caller's G, or the residual),
+  // without it off the output (the caller's U)
+  const int sb = sc.ex ? (int)(t % sc.batch) : 0;
+  const int ein = sc.ex && sc.G ? sc.ex[sb] : 0, eout = sc.ex && !sc.G ? -sc.ex[sb] : 0;
+  const bool dead = sc.ex && !sc.G && sc.zero[sb];
+  if (sc.G) {
+    rin.G = global_ptr(sc.G);
+    if constexpr (sizeof(Tin) == 8) X = global_ptr(sc.G);
+  }
   const Tin *Xt = X + t * ny * nx;
   Tout *Yt = Y + t * ny * nx;
   const int np = TX >> 1;
@@ -519,7 +556,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 5 : 1) k_dst_y(const Tin
     const int64_t tt = t / rin.batch;                // time step
     const int b = (int)(t - tt * rin.batch);         // problem
     const int64_t nb = (int64_t)rin.ny * nx;         // unknowns per time row
-    const double msc = rin.mex ? ldexp(1.0, rin.mex[b]) : 1.0;
+    const int rex = ein + (rin.mex ? rin.mex[b] : 0);
     for (int i0 = threadIdx.x; i0 < total; i0 += kLoadBatch * blockDim.x) {
       double rv[kLoadBatch];
 #pragma unroll
@@ -547,7 +584,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 5 : 1) k_dst_y(const Tin
 #pragma unroll
       for (int u = 0; u < kLoadBatch; ++u) {
         const int idx = i0 + u * (int)blockDim.x;
-        if (idx < total) rt[idx] = cvt<T>(rin.mex ? rv[u] * msc : rv[u]);
+        if (idx < total) rt[idx] = slot_load<T>(rv[u], rex);
       }
     }
     __syncthreads();
@@ -557,7 +594,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 5 : 1) k_dst_y(const Tin
     if constexpr (RES)
       return rt[y * TX + (int)(col - x0)];
     else
-      return cvt<T>(Xt[(int64_t)y * nx + col]);
+      return in_load<true, T>(Xt[(int64_t)y * nx + col], ein);
   };
   if constexpr (R16) {  // radix-16 first stage in registers (see k_fft_r2c16)
     const int SS = series_stride16(N), nb = N >> 4, lb = logN - 4, half = N >> 1;
@@ -634,11 +671,13 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 5 : 1) k_dst_y(const Tin
                            : buf[(size_t)(c >> 1) * series_stride(N) + l + 1];
       const T v = ((c & 1) == 0) ? (T(-0.5) * scale) * z.y : (T(0.5) * scale) * z.x;
       const int64_t o = (int64_t)l * nx + col;
-      if (mode == 0) {
-        Yt[o] = cvt<Tout>(v);
-      } else {
-        Yt[o] = old[u] + cvt<Tout>(v);
-      }
+      Tout d;
+      if constexpr (sizeof(Tout) == 8)
+        d = slot_store(v, eout);
+      else
+        d = v;
+      if (mode != 0) d = old[u] + d;
+      Yt[o] = dead ? Tout(0) : d;
     }
   }
 }
@@ -695,7 +734,7 @@ static int pick_tx(const Ctx &c, int n, int cap, int64_t ncols, int req = 0) {
 
 template <typename T, typename Tin>
 void launch_fft_r2c(Ctx &c, const Tin *X, int64_t ldx, int64_t ncols, int n, const cpx<T> *tw,
-                    cpx<T> *S, int64_t lds, const T *rs, const RhsNorm *rnp) {
+                    cpx<T> *S, int64_t lds, const T *rs, const RhsNorm *rnp, const SlotScale &sc) {
   const RhsNorm rn = rnp ? *rnp : RhsNorm{nullptr, nullptr, nullptr};
   const int logn = ilog2(n);
   const int TX = pick_tx<T>(c, n, sizeof(T) == 8 ? 8 : 16, ncols, c.fft_cols);
@@ -703,21 +742,20 @@ void launch_fft_r2c(Ctx &c, const Tin *X, int64_t ldx, int64_t ncols, int n, con
   const int grid = (int)((ncols + TX - 1) / TX);
   const double bytes = (double)n * ncols * sizeof(Tin) + (double)(n / 2 + 1) * ncols * sizeof(cpx<T>);
   if (rfft_built<T>(c, n, ncols))
-    return rfft_launch<T, Tin>(c, X, ldx, ncols, n, tw, S, lds, rs, rn,
-                                      sizeof(T) == 8 ? "fft_r2c_f64" : "fft_r2c_f32", bytes);
+    return rfft_launch<T, Tin>(c, X, ldx, ncols, n, tw, S, lds, rs, rn, sc,
+                               sizeof(T) == 8 ? "fft_r2c_f64" : "fft_r2c_f32", bytes);
   c.launch(sizeof(T) == 8 ? "fft_r2c_f64" : "fft_r2c_f32", bytes, [&] {
     PD_TX_DISPATCH(TX, {
       if (use_r16<T>(c, n)) {
         const int thr = fft16_threads((kTX / 2) * (n / 16), 512);
-        if (smem > 48 * 1024)
-          allow_dyn_smem((const void *)k_fft_r2c16<T, Tin, kTX>);
-        pdl_launch(c.pdl, k_fft_r2c16<T, Tin, kTX>, dim3(grid), dim3(thr), smem, c.stream, X, ldx, ncols, n, logn, tw,
-                   S, lds, rs, rn);
+        auto kern = sc.ex ? k_fft_r2c16<T, Tin, kTX, true> : k_fft_r2c16<T, Tin, kTX, false>;
+        if (smem > 48 * 1024) allow_dyn_smem((const void *)kern);
+        pdl_launch(c.pdl, kern, dim3(grid), dim3(thr), smem, c.stream, X, ldx, ncols, n, logn, tw, S, lds, rs, rn, sc);
       } else {
-        if (smem > 48 * 1024)
-          allow_dyn_smem((const void *)k_fft_r2c<T, Tin, kTX>);
-        pdl_launch(c.pdl, k_fft_r2c<T, Tin, kTX>, dim3(grid), dim3(fft_threads(n, kTX)), smem, c.stream, X, ldx, ncols,
-                   n, logn, tw, S, lds, rs, rn);
+        auto kern = sc.ex ? k_fft_r2c<T, Tin, kTX, true> : k_fft_r2c<T, Tin, kTX, false>;
+        if (smem > 48 * 1024) allow_dyn_smem((const void *)kern);
+        pdl_launch(c.pdl, kern, dim3(grid), dim3(fft_threads(n, kTX)), smem, c.stream, X, ldx, ncols, n, logn, tw, S, lds,
+                   rs, rn, sc);
       }
     })
   });
@@ -726,7 +764,7 @@ void launch_fft_r2c(Ctx &c, const Tin *X, int64_t ldx, int64_t ncols, int n, con
 template <typename T>
 void launch_fft_r2c_residual(Ctx &c, const double *G, const double *U, int64_t ncols, int n, const double *rxl,
                              const double *rxd, const double *rxu, const cpx<T> *tw, cpx<T> *S, int64_t lds,
-                             const T *rs, const int *mex, int mnx, const RhsNorm *rnp) {
+                             const T *rs, const int *mex, int mnx, const RhsNorm *rnp, const SlotScale &sc) {
   const RhsNorm rn = rnp ? *rnp : RhsNorm{nullptr, nullptr, nullptr};
   const int logn = ilog2(n);
   const int TX = pick_tx<T>(c, n, sizeof(T) == 8 ? 8 : 16, ncols, c.fft_cols);
@@ -735,10 +773,10 @@ void launch_fft_r2c_residual(Ctx &c, const double *G, const double *U, int64_t n
   const double bytes = (double)n * ncols * 16.0 + (double)(n / 2 + 1) * ncols * sizeof(cpx<T>);
   c.launch(sizeof(T) == 8 ? "fft_r2c_res_f64" : "fft_r2c_res_f32", bytes, [&] {
     PD_TX_DISPATCH(TX, {
-      if (smem > 48 * 1024)
-        allow_dyn_smem((const void *)k_fft_r2c_res<T, kTX>);
-      pdl_launch(c.pdl, k_fft_r2c_res<T, kTX>, dim3(grid), dim3(fft_threads(n, kTX)), smem, c.stream, G, U, ncols, n,
-                 logn, rxl, rxd, rxu, tw, S, lds, rs, mex, mnx, rn);
+      auto kern = sc.ex ? k_fft_r2c_res<T, kTX, true> : k_fft_r2c_res<T, kTX, false>;
+      if (smem > 48 * 1024) allow_dyn_smem((const void *)kern);
+      pdl_launch(c.pdl, kern, dim3(grid), dim3(fft_threads(n, kTX)), smem, c.stream, G, U, ncols, n,
+                 logn, rxl, rxd, rxu, tw, S, lds, rs, mex, mnx, rn, sc);
     })
   });
 }
@@ -746,7 +784,7 @@ void launch_fft_r2c_residual(Ctx &c, const double *G, const double *U, int64_t n
 template <typename T>
 void launch_fft_c2r(Ctx &c, const cpx<T> *S, int64_t lds, int64_t ncols, int n, const cpx<T> *tw,
                     void *out, int64_t ldo, int mode, double *norm_part, int *nparts, const StepFinish *finp,
-                    const T *rsi, double *colsum, const int *mex, int mnx, const int *skip) {
+                    const T *rsi, double *colsum, const int *mex, int mnx, const int *skip, const SlotScale &sc) {
   StepFinish fin{};
   if (finp && norm_part) fin = *finp;
   const int logn = ilog2(n);
@@ -757,21 +795,21 @@ void launch_fft_c2r(Ctx &c, const cpx<T> *S, int64_t lds, int64_t ncols, int n, 
   const double obytes = (mode == 2) ? 4.0 : (mode == 1 ? 16.0 : 8.0);
   const double bytes = (double)(n / 2 + 1) * ncols * sizeof(cpx<T>) + (double)n * ncols * obytes;
   if (rfft_built<T>(c, n, ncols))
-    return crfft_launch<T>(c, S, lds, ncols, n, tw, out, ldo, mode, norm_part, nparts, fin, rsi, colsum, mex, mnx, skip,
+    return crfft_launch<T>(c, S, lds, ncols, n, tw, out, ldo, mode, norm_part, nparts, fin, rsi, colsum, mex, mnx, skip, sc,
                            sizeof(T) == 8 ? "fft_c2r_f64" : "fft_c2r_f32", bytes);
   c.launch(sizeof(T) == 8 ? "fft_c2r_f64" : "fft_c2r_f32", bytes, [&] {
     PD_TX_DISPATCH(TX, {
       if (use_r16<T>(c, n)) {
         const int thr = fft16_threads((kTX / 2) * (n / 16), 256);
-        if (smem > 48 * 1024)
-          allow_dyn_smem((const void *)k_fft_c2r<T, kTX, true>);
-        pdl_launch(c.pdl, k_fft_c2r<T, kTX, true>, dim3(grid), dim3(thr), smem, c.stream, S, lds, ncols, n, logn, tw, out,
-                   ldo, mode, norm_part, fin, rsi, colsum, mex, mnx, skip);
+        auto kern = sc.ex ? k_fft_c2r<T, kTX, true, true> : k_fft_c2r<T, kTX, true, false>;
+        if (smem > 48 * 1024) allow_dyn_smem((const void *)kern);
+        pdl_launch(c.pdl, kern, dim3(grid), dim3(thr), smem, c.stream, S, lds, ncols, n, logn, tw, out, ldo, mode, norm_part,
+                   fin, rsi, colsum, mex, mnx, skip, sc);
       } else {
-        if (smem > 48 * 1024)
-          allow_dyn_smem((const void *)k_fft_c2r<T, kTX, false>);
-        pdl_launch(c.pdl, k_fft_c2r<T, kTX, false>, dim3(grid), dim3(256), smem, c.stream, S, lds, ncols, n, logn, tw,
-                   out, ldo, mode, norm_part, fin, rsi, colsum, mex, mnx, skip);
+        auto kern = sc.ex ? k_fft_c2r<T, kTX, false, true> : k_fft_c2r<T, kTX, false, false>;
+        if (smem > 48 * 1024) allow_dyn_smem((const void *)kern);
+        pdl_launch(c.pdl, kern, dim3(grid), dim3(256), smem, c.stream, S, lds, ncols, n, logn, tw, out, ldo, mode, norm_part,
+                   fin, rsi, colsum, mex, mnx, skip, sc);
       }
     })
   });
@@ -779,10 +817,10 @@ void launch_fft_c2r(Ctx &c, const cpx<T> *S, int64_t lds, int64_t ncols, int n, 
 
 template <typename Tin, typename Tout, typename T, bool RES>
 static void dst_launch(Ctx &c, const Tin *X, Tout *Y, int64_t nslab, int64_t ny, int64_t nx, const cpx<T> *tw,
-                       int mode, const int *skip, const ResIn &rin, const char *fam, double bytes) {
+                       int mode, const int *skip, const ResIn &rin, const SlotScale &sc, const char *fam, double bytes) {
   // the half-extension kernel where it is the faster one, unless the caller chose a first-stage radix
-  if (c.fft_radix == 0 && dst2_fits(ny, nslab * nx, RES && sizeof(T) == 4))
-    return launch_dst2<Tin, Tout, T, RES>(c, X, Y, nslab * nx, ny, nx, tw, mode, skip, rin, fam, bytes);
+  if (c.fft_radix == 0 && !(sc.ex && ny == 255) && dst2_fits(ny, nslab * nx, RES && sizeof(T) == 4))
+    return launch_dst2<Tin, Tout, T, RES>(c, X, Y, nslab * nx, ny, nx, tw, mode, skip, rin, sc, fam, bytes);
   const int N = (int)(2 * (ny + 1));
   const int logN = ilog2(N);
   const int TX = pick_tx<T>(c, N, sizeof(T) == 8 ? 8 : 16, nslab * nx);
@@ -798,12 +836,12 @@ static void dst_launch(Ctx &c, const Tin *X, Tout *Y, int64_t nslab, int64_t ny,
         if (smem > 48 * 1024)
           allow_dyn_smem((const void *)k_dst_y<Tin, Tout, T, kTX, true, RES>);
         pdl_launch(c.pdl, k_dst_y<Tin, Tout, T, kTX, true, RES>, dim3((unsigned)grid), dim3(256), smem, c.stream, X, Y,
-                   ny, nx, N, logN, tw, scale, mode, skip, rin, res_off);
+                   ny, nx, N, logN, tw, scale, mode, skip, rin, res_off, sc);
       } else {
         if (smem > 48 * 1024)
           allow_dyn_smem((const void *)k_dst_y<Tin, Tout, T, kTX, false, RES>);
         pdl_launch(c.pdl, k_dst_y<Tin, Tout, T, kTX, false, RES>, dim3((unsigned)grid), dim3(256), smem, c.stream, X,
-                   Y, ny, nx, N, logN, tw, scale, mode, skip, rin, res_off);
+                   Y, ny, nx, N, logN, tw, scale, mode, skip, rin, res_off, sc);
       }
     })
   });
@@ -811,54 +849,54 @@ static void dst_launch(Ctx &c, const Tin *X, Tout *Y, int64_t nslab, int64_t ny,
 
 template <typename Tin, typename Tout, typename T>
 void launch_dst_y(Ctx &c, const Tin *X, Tout *Y, int64_t nt, int64_t ny, int64_t nx, const cpx<T> *tw,
-                  int mode, const int *skip) {
+                  int mode, const int *skip, const SlotScale &sc) {
   const double bytes = (double)nt * ny * nx * (sizeof(Tin) + sizeof(Tout) * (mode ? 2 : 1));
-  dst_launch<Tin, Tout, T, false>(c, X, Y, nt, ny, nx, tw, mode, skip, ResIn{}, sizeof(T) == 8 ? "dst_y_f64" : "dst_y_f32",
-                                  bytes);
+  dst_launch<Tin, Tout, T, false>(c, X, Y, nt, ny, nx, tw, mode, skip, ResIn{}, sc,
+                                  sizeof(T) == 8 ? "dst_y_f64" : "dst_y_f32", bytes);
 }
 
 template <typename T>
 void launch_dst_y_residual(Ctx &c, const double *G, const double *U, T *Y, int64_t nt, int batch, int64_t nym,
                            int64_t nx, const double *rxl, const double *rdd, const double *rxu, const double *ryl,
-                           const double *ryu, const int *mex, const cpx<T> *tw) {
+                           const double *ryu, const int *mex, const cpx<T> *tw, const SlotScale &sc) {
   ResIn rin{G, U, rxl, rdd, rxu, ryl, ryu, (int)(nym * batch), (int)nym, batch, mex};
   // G and U read once (neighbours from the caches), the binary32 / FP64 transform written
   const double bytes = (double)nt * batch * nym * nx * (16.0 + sizeof(T));
-  dst_launch<double, T, T, true>(c, (const double *)nullptr, Y, nt * batch, nym, nx, tw, 0, nullptr, rin,
+  dst_launch<double, T, T, true>(c, (const double *)nullptr, Y, nt * batch, nym, nx, tw, 0, nullptr, rin, sc,
                                  sizeof(T) == 8 ? "dst_y_res_f64" : "dst_y_res_f32", bytes);
 }
 
 template void launch_fft_r2c<double, double>(Ctx &, const double *, int64_t, int64_t, int, const cpx<double> *,
-                                             cpx<double> *, int64_t, const double *, const RhsNorm *);
+                                             cpx<double> *, int64_t, const double *, const RhsNorm *, const SlotScale &);
 template void launch_fft_r2c<float, double>(Ctx &, const double *, int64_t, int64_t, int, const cpx<float> *,
-                                            cpx<float> *, int64_t, const float *, const RhsNorm *);
+                                            cpx<float> *, int64_t, const float *, const RhsNorm *, const SlotScale &);
 template void launch_fft_r2c<float, float>(Ctx &, const float *, int64_t, int64_t, int, const cpx<float> *,
-                                           cpx<float> *, int64_t, const float *, const RhsNorm *);
+                                           cpx<float> *, int64_t, const float *, const RhsNorm *, const SlotScale &);
 template void launch_fft_c2r<double>(Ctx &, const cpx<double> *, int64_t, int64_t, int, const cpx<double> *,
                                      void *, int64_t, int, double *, int *, const StepFinish *, const double *,
-                                     double *, const int *, int, const int *);
+                                     double *, const int *, int, const int *, const SlotScale &);
 template void launch_fft_c2r<float>(Ctx &, const cpx<float> *, int64_t, int64_t, int, const cpx<float> *,
                                     void *, int64_t, int, double *, int *, const StepFinish *, const float *,
-                                    double *, const int *, int, const int *);
+                                    double *, const int *, int, const int *, const SlotScale &);
 template void launch_fft_r2c_residual<double>(Ctx &, const double *, const double *, int64_t, int, const double *,
                                               const double *, const double *, const cpx<double> *, cpx<double> *,
-                                              int64_t, const double *, const int *, int, const RhsNorm *);
+                                              int64_t, const double *, const int *, int, const RhsNorm *, const SlotScale &);
 template void launch_fft_r2c_residual<float>(Ctx &, const double *, const double *, int64_t, int, const double *,
                                              const double *, const double *, const cpx<float> *, cpx<float> *,
-                                             int64_t, const float *, const int *, int, const RhsNorm *);
+                                             int64_t, const float *, const int *, int, const RhsNorm *, const SlotScale &);
 template void launch_dst_y<double, double, double>(Ctx &, const double *, double *, int64_t, int64_t, int64_t,
-                                                   const cpx<double> *, int, const int *);
+                                                   const cpx<double> *, int, const int *, const SlotScale &);
 template void launch_dst_y<double, float, float>(Ctx &, const double *, float *, int64_t, int64_t, int64_t,
-                                                 const cpx<float> *, int, const int *);
+                                                 const cpx<float> *, int, const int *, const SlotScale &);
 template void launch_dst_y<float, float, float>(Ctx &, const float *, float *, int64_t, int64_t, int64_t,
-                                                const cpx<float> *, int, const int *);
+                                                const cpx<float> *, int, const int *, const SlotScale &);
 template void launch_dst_y<float, double, float>(Ctx &, const float *, double *, int64_t, int64_t, int64_t,
-                                                 const cpx<float> *, int, const int *);
+                                                 const cpx<float> *, int, const int *, const SlotScale &);
 template void launch_dst_y_residual<float>(Ctx &, const double *, const double *, float *, int64_t, int, int64_t,
                                            int64_t, const double *, const double *, const double *, const double *,
-                                           const double *, const int *, const cpx<float> *);
+                                           const double *, const int *, const cpx<float> *, const SlotScale &);
 template void launch_dst_y_residual<double>(Ctx &, const double *, const double *, double *, int64_t, int, int64_t,
                                             int64_t, const double *, const double *, const double *, const double *,
-                                            const double *, const int *, const cpx<double> *);
+                                            const double *, const int *, const cpx<double> *, const SlotScale &);
 
 }  // namespace pd

@@ -93,12 +93,15 @@ __device__ __forceinline__ void team_sync(int P, int team_in_cta) {
 // DST).  The significand is truncated (error below one binary32 ulp, where round-to-nearest
 // gives half an ulp); magnitudes below binary32's normal range become zero, above it
 // infinity; NaN stays NaN.
-__device__ __forceinline__ float f64_to_f32_bits(double x) {
+// SCALE: the value times 2^k (|k| < 1000).
+template <bool SCALE = false>
+__device__ __forceinline__ float f64_to_f32_bits(double x, int k = 0) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
   const unsigned hi = (unsigned)(b >> 32), lo = (unsigned)b;
   const unsigned sign = hi & 0x80000000u;
   const int e = (int)((hi >> 20) & 0x7ffu);
-  const int ef = e - 896;  // binary32 biased exponent: e - 1023 + 127
+  int ef = e - 896;  // binary32 biased exponent: e - 1023 + 127
+  if constexpr (SCALE) ef = e == 0 ? 0 : e == 0x7ff ? 255 : ef + k;
   unsigned r;
   if (ef >= 255) {
     r = sign | 0x7f800000u | ((e == 0x7ff && ((hi & 0xfffffu) | lo)) ? 0x00400000u : 0u);
@@ -111,10 +114,11 @@ __device__ __forceinline__ float f64_to_f32_bits(double x) {
 }
 // binary32 -> binary64 by integer operations, for the same reason (the stores of the inverse
 // transforms: one conversion beside the one FP64 add of U += delta).  Exact for normal numbers
-// and infinities; subnormals become zero, NaN stays NaN.
-__device__ __forceinline__ double f32_to_f64_bits(float x) {
+// and infinities; subnormals become zero, NaN stays NaN.  k: times 2^k, |k| <= 800 (every binary32
+// number then stays normal in binary64).
+__device__ __forceinline__ double f32_to_f64_bits(float x, int k = 0) {
   const unsigned b = __float_as_uint(x), m = b & 0x7fffffffu;
-  unsigned hi = (m >> 3) + (m >= 0x7f800000u ? 0x70000000u : 0x38000000u);  // exponent + 896 (+ 1792)
+  unsigned hi = (m >> 3) + (m >= 0x7f800000u ? 0x70000000u : 0x38000000u + ((unsigned)k << 20));  // exponent + 896 + k
   unsigned lo = m << 29;
   if (m < 0x00800000u) hi = lo = 0u;
   return __hiloint2double((int)(hi | (b & 0x80000000u)), (int)lo);
@@ -130,14 +134,42 @@ __device__ __forceinline__ To cvt(From x) {
     return (To)x;
 }
 
-// x * 2^k exactly: an exponent-field add for normal x whose result stays normal
-// (zero stays zero); other cases (subnormal, overflow, Inf/NaN) take ldexp.
+// x * 2^k by an exponent-field add (|k| < 1000): exact where the result is a normal number; below
+// that, zero; zero, infinities and NaN stay.  The batches' scale factors come from sums of squares
+// in binary64, so their exponents lie within +-540 and the rest of a problem far above that floor.
 __device__ __forceinline__ double pow2_scale(double x, int k) {
-  const long long bits = __double_as_longlong(x);
-  if ((bits & 0x7fffffffffffffffLL) == 0) return x;
-  const int e = (int)((bits >> 52) & 0x7ff);
-  if (e > 0 && e < 0x7ff && e + k > 0 && e + k < 0x7ff) return __longlong_as_double(bits + ((long long)k << 52));
-  return ldexp(x, k);
+  const int hi = __double2hiint(x), e = (hi >> 20) & 0x7ff, t = e + k;
+  int h = hi + (k << 20), l = __double2loint(x);
+  if (t >= 0x7ff) {  // overflow: infinity
+    h = (hi & 0x80000000) | 0x7ff00000;
+    l = 0;
+  }
+  if (e == 0 || t <= 0) {
+    h = hi & 0x80000000;
+    l = 0;
+  }
+  return e == 0x7ff ? x : __hiloint2double(h, l);
+}
+// Problem scaling of the batches on load and store: x 2^k in type T, and back to binary64.
+template <typename T>
+__device__ __forceinline__ T slot_load(double x, int k) {
+  if constexpr (sizeof(T) == 4)
+    return f64_to_f32_bits<true>(x, k);
+  else
+    return k ? pow2_scale(x, k) : x;
+}
+template <typename T>
+__device__ __forceinline__ double slot_store(T x, int k) {
+  if constexpr (sizeof(T) == 4)
+    return f32_to_f64_bits(x, k);
+  else
+    return k ? pow2_scale(x, k) : x;
+}
+// A pointer read from memory, known to be a global address (so that loads through it are global loads).
+__device__ __forceinline__ const double *global_ptr(const double *const *p) {
+  const double *q = *p;
+  __builtin_assume(__isGlobal(q));
+  return q;
 }
 
 // Programmatic dependent launch: every kernel of this library opens with this wait,

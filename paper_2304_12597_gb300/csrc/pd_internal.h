@@ -165,9 +165,21 @@ struct RhsNorm {
   int *counter;  // zero on entry; reset by the last CTA
   double *dst;
 };
+// Batched plans: problem b (columns [b mnx, (b+1) mnx) in 1D, slabs s with s mod batch = b in 2D) is
+// solved scaled to unit norm by the exact factor 2^ex[b].  The transforms apply it where they load
+// the caller's right-hand side and undo it where they store the caller's solution, so that neither
+// array is passed over for it.  All null for single problems.
+struct SlotScale {
+  const int *ex = nullptr;
+  const int *zero = nullptr;         // all-zero problems: their solution is stored as exact zeros
+  const int *nxb = nullptr;          // 1D: rows of each problem; columns past them are stored as exact zeros
+  const double *const *G = nullptr;  // the caller's right-hand side (written per solve, read by the graph)
+  int mnx = 1, batch = 1;
+};
 template <typename T, typename Tin>
 void launch_fft_r2c(Ctx &c, const Tin *X, int64_t ldx, int64_t ncols, int n, const cpx<T> *tw,
-                    cpx<T> *S, int64_t lds, const T *rs = nullptr, const RhsNorm *rn = nullptr);
+                    cpx<T> *S, int64_t lds, const T *rs = nullptr, const RhsNorm *rn = nullptr,
+                    const SlotScale &sc = {});
 // Forward DFT along time of the FP64 all-at-once residual
 // R = G - [(I + tau K) U - U Sigma_1^T] (1D), computed on load: R is never stored.
 // mex/mnx (batched plans): column c is scaled by 2^mex[c / mnx], undone by the inverse.
@@ -175,7 +187,7 @@ template <typename T>
 void launch_fft_r2c_residual(Ctx &c, const double *G, const double *U, int64_t ncols, int n,
                              const double *rxl, const double *rxd, const double *rxu, const cpx<T> *tw,
                              cpx<T> *S, int64_t lds, const T *rs = nullptr, const int *mex = nullptr,
-                             int mnx = 1, const RhsNorm *rn = nullptr);
+                             int mnx = 1, const RhsNorm *rn = nullptr, const SlotScale &sc = {});
 // Optional epilogue of the inverse DFT: the last CTA to finish sums the per-CTA
 // squares into scal[S_D2] and runs the refinement decision.
 struct StepFinish {
@@ -199,11 +211,11 @@ bool rfft_built(const Ctx &c, int n, int64_t ncols) {
 }
 template <typename T, typename Tin>
 void rfft_launch(Ctx &c, const Tin *X, int64_t ldx, int64_t ncols, int n, const cpx<T> *tw, cpx<T> *S, int64_t lds,
-                 const T *rs, const RhsNorm &rn, const char *fam, double bytes);
+                 const T *rs, const RhsNorm &rn, const SlotScale &sc, const char *fam, double bytes);
 template <typename T>
 void crfft_launch(Ctx &c, const cpx<T> *S, int64_t lds, int64_t ncols, int n, const cpx<T> *tw, void *out, int64_t ldo,
                   int mode, double *norm_part, int *nparts, const StepFinish &fin, const T *rsi, double *colsum,
-                  const int *mex, int mnx, const int *skip, const char *fam, double bytes);
+                  const int *mex, int mnx, const int *skip, const SlotScale &sc, const char *fam, double bytes);
 // Inverse DFT along time of a half spectrum; mode 0: store double, 1: add into
 // double, 2: store float.  norm_part (may be null) receives per-CTA sums of the
 // squared output values; *nparts = number of CTAs.  colsum (may be null) receives
@@ -212,7 +224,7 @@ template <typename T>
 void launch_fft_c2r(Ctx &c, const cpx<T> *S, int64_t lds, int64_t ncols, int n, const cpx<T> *tw,
                     void *out, int64_t ldo, int mode, double *norm_part, int *nparts,
                     const StepFinish *fin = nullptr, const T *rsi = nullptr, double *colsum = nullptr,
-                    const int *mex = nullptr, int mnx = 1, const int *skip = nullptr);
+                    const int *mex = nullptr, int mnx = 1, const int *skip = nullptr, const SlotScale &sc = {});
 // The FP64 all-at-once residual as the DST's input (ResIn.G != null): element (row y, column
 // col) of slab s (time t = s / batch, problem b = s % batch) is
 // r = G_t + u_{t-1} - [(I + tau T_x) u_t + tau T_y u_t] at row b nym + y of the stacked grid
@@ -231,12 +243,12 @@ struct ResIn {
 bool dst2_fits(int64_t ny, int64_t ncol, bool res_f32);
 template <typename Tin, typename Tout, typename T, bool RES>
 void launch_dst2(Ctx &c, const Tin *X, Tout *Y, int64_t ncol, int64_t ny, int64_t nx, const cpx<T> *tw, int mode,
-                 const int *skip, const ResIn &rin, const char *fam, double bytes);
+                 const int *skip, const ResIn &rin, const SlotScale &sc, const char *fam, double bytes);
 // Orthonormal DST-I along the middle axis of (nt, ny, nx); ny + 1 a power of two.
 // mode 0: store, 1: add into (double output only).
 template <typename Tin, typename Tout, typename T>
 void launch_dst_y(Ctx &c, const Tin *X, Tout *Y, int64_t nt, int64_t ny, int64_t nx,
-                  const cpx<T> *tw, int mode, const int *skip = nullptr);
+                  const cpx<T> *tw, int mode, const int *skip = nullptr, const SlotScale &sc = {});
 // The same transform of the FP64 all-at-once residual of the 2D path, formed while each tile
 // loads (nt time rows of batch problems, nym rows of T_y each, stacked along y; rx
 // per problem, ry over the stacked rows; mex: the batches' residual scaling, or null):
@@ -245,7 +257,7 @@ void launch_dst_y(Ctx &c, const Tin *X, Tout *Y, int64_t nt, int64_t ny, int64_t
 template <typename T>
 void launch_dst_y_residual(Ctx &c, const double *G, const double *U, T *Y, int64_t nt, int batch, int64_t nym,
                            int64_t nx, const double *rxl, const double *rdd, const double *rxu, const double *ryl,
-                           const double *ryu, const int *mex, const cpx<T> *tw);
+                           const double *ryu, const int *mex, const cpx<T> *tw, const SlotScale &sc = {});
 
 // ---- the operator's device arrays (operator.cu) ---------------------------------------
 struct OperatorArgs {
@@ -350,20 +362,15 @@ struct ProjTail;  // pd_krylov.cuh: eq. 13 and the step decision run by the z re
 template <typename T>
 void launch_zsum(Ctx &c, int nf, int64_t n, const cpx<T> *H, int64_t ldh, const double2 *omega, double *z,
                  const int *skip_flag, const ProjTail *tail = nullptr, int mlen = 0, const double *h0 = nullptr);
-// Batched plans (batch.cu): Gs = G with slot b scaled by 2^ex[b] ~ 1/||slot b||_F
-// (part: batch * nc doubles of scratch; zero[b] = 1 marks an all-zero slot), and the
-// inverse scaling of U in place with the columns past problem b's nxb[b] rows, and every
-// column of an all-zero problem, set to zero.
-void launch_batch_normalize(Ctx &c, const double *G, double *Gs, int64_t nt, int batch, int nxm, int nc,
-                            double *part, int *ex, int *zero);
+// Batched plans (batch.cu): the scale exponents ex[b] = -round(log2 ||slot b||_F) of the right-hand
+// side G (part: batch * nc doubles of scratch; zero[b] = 1 marks an all-zero slot), and *gslot = G.
+void launch_batch_exponents(Ctx &c, const double *G, int64_t nt, int batch, int nxm, int nc, double *part, int *ex,
+                            int *zero, const double **gslot);
 // Problems joining a running batched solve (paradiag_batch_advance): for join[b] != 0 the
 // slot's U is zeroed and its refinement state reset (msw, mprev, mref2, mex, mconv); unused
-// slots (zero[b]) start from U = 0 as well; the other slots' U is scaled by 2^ex[b] into
-// the solve's units (exact).
-void launch_member_join(Ctx &c, double *U, int64_t nt, int batch, int nxm, const int *ex, const int *join,
-                        const int *zero, int *msw, double *prev, double *ref2, int *mex, int *mconv);
-void launch_batch_unscale(Ctx &c, double *U, int64_t nt, int batch, int nxm, const int *ex, const int *nxb,
-                          const int *zero);
+// slots (zero[b]) start from U = 0 as well.
+void launch_member_join(Ctx &c, double *U, int64_t nt, int batch, int nxm, const int *join, const int *zero, int *msw,
+                        double *prev, double *ref2, int *mex, int *mconv);
 // out[t][j] = in[t][j] * s[j] over nt rows of nb columns (in place allowed; batch.cu)
 void launch_col_scale(Ctx &c, const double *in, double *out, int64_t nt, int64_t nb, const double *s);
 // Batched plans: per-problem ||delta||^2 from the inverse DFT's per-column sums, then the

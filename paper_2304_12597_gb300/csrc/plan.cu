@@ -212,7 +212,7 @@ struct pd_plan {
   int64_t nxd = 0;   // the descriptor's nx
   int64_t nxm = 0;
   int bnc = 0;                  // time-row groups of the per-problem norm pass
-  double *Gs = nullptr;         // G with every problem scaled to unit norm
+  const double **gslot = nullptr;  // device: the right-hand side of the solve in progress
   double *bpart = nullptr;      // norm partials (batch * bnc)
   int *bex = nullptr;           // per-problem power-of-two scale exponents
   int *bzero = nullptr;         // per-problem flag: all-zero right-hand side (unused slot)
@@ -736,7 +736,7 @@ size_t layout(pd_plan *p, unsigned char *base) {
     p->Gm = A.take<double>((size_t)nt * nbar);
   }
   if (p->batch > 1) {
-    p->Gs = A.take<double>((size_t)nt * nbar);
+    p->gslot = A.take<const double *>(1);
     p->bpart = A.take<double>((size_t)p->batch * p->bnc);
     p->bex = A.take<int>(p->batch);
     p->bzero = A.take<int>(p->batch);
@@ -1171,6 +1171,20 @@ pd::KrylovCtl krylov_ctl(pd_plan *p, int kind) {
   return k;
 }
 
+// The batches' exact scaling between the caller's G and U and the solve: on load of G (in) or on
+// store of U.
+pd::SlotScale slot_scale(const pd_plan *p, bool in) {
+  pd::SlotScale s;
+  if (p->batch < 2) return s;
+  s.ex = p->bex;
+  s.zero = p->bzero;
+  s.nxb = p->bnx;
+  s.G = in ? p->gslot : nullptr;
+  s.mnx = (int)p->nxm;
+  s.batch = p->batch;
+  return s;
+}
+
 pd::RefineCtl refine_ctl(pd_plan *p) {
   const bool fp64 = p->precision == PD_FP64;
   pd::RefineCtl r;
@@ -1210,20 +1224,22 @@ pd_status emit_pre(pd_plan *p, int kind, const double *G, double *U, int use_han
   const pd::RhsNorm *rnp = p->members ? nullptr : &rn;
   if (kind == 0) {
     if (p->dim == 1) {
-      pd::launch_fft_r2c<T, double>(c, G, p->nbar, p->nbar, nt, time_tw<T>(p), S, p->lds, row_scale<T>(p, false),
-                                    rnp);
+      pd::launch_fft_r2c<T, double>(c, G, p->nbar, p->nbar, nt, time_tw<T>(p), S, p->lds, row_scale<T>(p, false), rnp,
+                                    slot_scale(p, true));
     } else {
-      pd::launch_dst_y<double, T, T>(c, G, tmp, p->nt * p->batch, p->nym, p->nx, dst_tw<T>(p), 0);
+      pd::launch_dst_y<double, T, T>(c, G, tmp, p->nt * p->batch, p->nym, p->nx, dst_tw<T>(p), 0, nullptr,
+                                     slot_scale(p, true));
       pd::launch_fft_r2c<T, T>(c, tmp, p->nbar, p->nbar, nt, time_tw<T>(p), S, p->lds, row_scale<T>(p, false), rnp);
     }
   } else {
     if (p->dim == 1) {  // the FP64 residual is formed while the DFT loads its tiles
       pd::launch_fft_r2c_residual<T>(c, G, U, p->nbar, nt, p->rxl, p->rxd, p->rxu, time_tw<T>(p), S, p->lds,
-                                     row_scale<T>(p, false), p->batch > 1 ? p->mex : nullptr, (int)p->nxm, rnp);
+                                     row_scale<T>(p, false), p->batch > 1 ? p->mex : nullptr, (int)p->nxm, rnp,
+                                     slot_scale(p, true));
     } else {
       // the FP64 residual is formed while the DST along y loads its tiles
       pd::launch_dst_y_residual<T>(c, G, U, tmp, p->nt, p->batch, p->nym, p->nx, p->rxl, p->rdd, p->rxu, p->ryl,
-                                   p->ryu, p->batch > 1 ? p->mex : nullptr, dst_tw<T>(p));
+                                   p->ryu, p->batch > 1 ? p->mex : nullptr, dst_tw<T>(p), slot_scale(p, true));
       pd::launch_fft_r2c<T, T>(c, tmp, p->nbar, p->nbar, nt, time_tw<T>(p), S, p->lds, row_scale<T>(p, false), rnp);
     }
   }
@@ -1428,11 +1444,12 @@ pd_status emit_post(pd_plan *p, int kind, double *U, int use_handle, cudaGraphCo
       T *tmp = tmp_buf<T>(p);
       pd::launch_fft_c2r<T>(c, S, p->lds, p->nbar, nt, time_tw<T>(p), tmp, p->nbar, fp64 ? 0 : 2, nullptr, &nparts,
                             nullptr, row_scale<T>(p, true), p->colsum, kind == 0 ? nullptr : p->mex, (int)p->nxm);
-      pd::launch_dst_y<T, double, T>(c, tmp, U, p->nt * p->batch, p->nym, p->nx, dst_tw<T>(p), kind == 0 ? 0 : 1);
+      pd::launch_dst_y<T, double, T>(c, tmp, U, p->nt * p->batch, p->nym, p->nx, dst_tw<T>(p), kind == 0 ? 0 : 1, nullptr,
+                                     slot_scale(p, false));
     } else {
       pd::launch_fft_c2r<T>(c, S, p->lds, p->nbar, nt, time_tw<T>(p), U, p->nbar, kind == 0 ? 0 : 1, nullptr,
                             &nparts, nullptr, row_scale<T>(p, true), p->colsum, kind == 0 ? nullptr : p->mex,
-                            (int)p->nxm);
+                            (int)p->nxm, nullptr, slot_scale(p, false));
     }
     pd::launch_member_decide(c, p->colsum, (int)p->nxm, p->bnx, p->batch, p->md2, p->mref2, p->mprev, p->mex, p->bzero,
                              p->scal, p->flags, refine_ctl(p), use_handle, hr);
@@ -1903,13 +1920,12 @@ pd_status paradiag_solve(pd_plan *p, const double *G, double *U, pd_stats *stats
     Gin = p->Gm;
   }
   if (p->batch > 1) {  // every problem of the batch scaled to unit norm (exactly, by 2^k)
-    pd::launch_batch_normalize(p->ctx, Gin, p->Gs, p->nt, p->batch, (int)p->nxm, p->bnc, p->bpart, p->bex, p->bzero);
-    Gin = p->Gs;
+    pd::launch_batch_exponents(p->ctx, Gin, p->nt, p->batch, (int)p->nxm, p->bnc, p->bpart, p->bex, p->bzero, p->gslot);
+    Gin = nullptr;  // (the transforms read it from gslot: the graph serves any right-hand side)
     CK(cudaMemsetAsync(p->msw, 0, sizeof(int) * p->batch, p->ctx.stream));  // every problem starts here
   }
   st = p->precision == PD_FP64 ? solve_refined<double>(p, Gin, U, s) : solve_refined<float>(p, Gin, U, s);
   if (st == PD_ERR_CUDA) return st;
-  if (p->batch > 1) pd::launch_batch_unscale(p->ctx, U, p->nt, p->batch, (int)p->nxm, p->bex, p->bnx, p->bzero);
   if (p->mass) pd::launch_col_scale(p->ctx, U, U, p->nt, p->nbar, p->msc);  // u = M^{-1/2} w
   CK(cudaEventRecord(p->ev1, p->ctx.stream));
   CK(cudaEventSynchronize(p->ev1));
@@ -1941,17 +1957,16 @@ pd_status paradiag_batch_advance(pd_plan *p, const double *G, double *U, const i
   const int64_t l0 = p->ctx.launches;
   CK(cudaEventRecord(p->ev0, p->ctx.stream));
   CK(cudaMemcpyAsync(p->mjoin, join, sizeof(int32_t) * p->batch, cudaMemcpyHostToDevice, p->ctx.stream));
-  pd::launch_batch_normalize(p->ctx, G, p->Gs, p->nt, p->batch, (int)p->nxm, p->bnc, p->bpart, p->bex, p->bzero);
-  pd::launch_member_join(p->ctx, U, p->nt, p->batch, (int)p->nxm, p->bex, p->mjoin, p->bzero, p->msw, p->mprev,
-                         p->mref2, p->mex, p->mconv);
+  pd::launch_batch_exponents(p->ctx, G, p->nt, p->batch, (int)p->nxm, p->bnc, p->bpart, p->bex, p->bzero, p->gslot);
+  pd::launch_member_join(p->ctx, U, p->nt, p->batch, (int)p->nxm, p->mjoin, p->bzero, p->msw, p->mprev, p->mref2, p->mex,
+                         p->mconv);
   const int keep_max = p->max_refine;
   p->max_refine = steps - 1;         // this call's sweeps
   p->member_solves = keep_max + 1;   // each problem's own limit, counted over calls
-  st = p->precision == PD_FP64 ? solve_continue<double>(p, p->Gs, U) : solve_continue<float>(p, p->Gs, U);
+  st = p->precision == PD_FP64 ? solve_continue<double>(p, nullptr, U) : solve_continue<float>(p, nullptr, U);
   p->max_refine = keep_max;
   p->member_solves = 0;
   if (st == PD_ERR_CUDA) return st;
-  pd::launch_batch_unscale(p->ctx, U, p->nt, p->batch, (int)p->nxm, p->bex, p->bnx, p->bzero);
   CK(cudaMemcpyAsync(state, p->mconv, sizeof(int32_t) * p->batch, cudaMemcpyDeviceToHost, p->ctx.stream));
   CK(cudaEventRecord(p->ev1, p->ctx.stream));
   CK(cudaEventSynchronize(p->ev1));

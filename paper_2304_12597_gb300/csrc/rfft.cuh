@@ -58,10 +58,10 @@ constexpr int rfft_ctas() {
 }
 
 // Forward transform of X (n, ldx).
-template <typename T, typename Tin, int R1, int R2, int TX>
+template <typename T, typename Tin, int R1, int R2, int TX, bool SLOT>
 __global__ void __launch_bounds__(rfft_threads<R1, R2, TX>(), rfft_ctas<T, R1, R2, TX>())
     k_rfft(const Tin *__restrict__ X, int64_t ldx, int64_t ncols, const cpx<T> *__restrict__ tw, cpx<T> *__restrict__ S,
-           int64_t lds, const T *__restrict__ rs, RhsNorm rn) {
+           int64_t lds, const T *__restrict__ rs, RhsNorm rn, SlotScale sc) {
   grid_dep_wait();
   constexpr int n = R1 * R2, H = R1 / 2 + 1, NIT = rfft_threads<R1, R2, TX>() / TX;
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -70,6 +70,11 @@ __global__ void __launch_bounds__(rfft_threads<R1, R2, TX>(), rfft_ctas<T, R1, R
   const int64_t col = (int64_t)blockIdx.x * TX + cl;
   const bool live = col < ncols;
   float ss = 0.0f;  // squares of the input (rn: a reference scale)
+  int ex = 0;
+  if constexpr (SLOT) {
+    X = global_ptr(sc.G);
+    if (live) ex = sc.ex[col / sc.mnx];
+  }
   for (int r = it0; r < R2; r += NIT) {
     T x[R1];
     constexpr int LB = R1 < 16 ? R1 : 16;  // rows whose loads are in flight together
@@ -79,7 +84,12 @@ __global__ void __launch_bounds__(rfft_threads<R1, R2, TX>(), rfft_ctas<T, R1, R
 #pragma unroll
       for (int i = 0; i < LB; ++i) v[i] = live ? X[(int64_t)(r + R2 * (i0 + i)) * ldx + col] : Tin(0);
 #pragma unroll
-      for (int i = 0; i < LB; ++i) x[i0 + i] = cvt<T>(v[i]);
+      for (int i = 0; i < LB; ++i) {
+        if constexpr (SLOT)
+          x[i0 + i] = slot_load<T>(v[i], ex);
+        else
+          x[i0 + i] = cvt<T>(v[i]);
+      }
     }
     if (rn.part) {
 #pragma unroll
@@ -124,12 +134,12 @@ __global__ void __launch_bounds__(rfft_threads<R1, R2, TX>(), rfft_ctas<T, R1, R
 // Inverse: X[j] = Re((1/n) sum_k w_n^{-jk} Y[k]) with Y[n - k] = conj Y[k], times rsi[j] and, for
 // batches, 2^-mex[col / mnx].  mode 0: store binary64, 1: add into binary64, 2: store binary32.
 // Everything runs on conjugates: the result is real, so x_j = sum_k conj(Y[k]) w^{jk} / n.
-template <typename T, int R1, int R2, int TX, int MODE>
+template <typename T, int R1, int R2, int TX, int MODE, bool SLOT>
 __global__ void __launch_bounds__(rfft_threads<R1, R2, TX>(), rfft_ctas<T, R1, R2, TX>())
     k_crfft(const cpx<T> *__restrict__ S, int64_t lds, int64_t ncols, const cpx<T> *__restrict__ tw,
             void *__restrict__ outv, int64_t ldo, double *__restrict__ norm_part, StepFinish fin,
             const T *__restrict__ rsi, double *__restrict__ colsum, const int *__restrict__ mex, int mnx,
-            const int *skip) {
+            const int *skip, SlotScale sc) {
   grid_dep_wait();
   if (skip && *skip) return;  // U already holds the result (Algorithm 3's U_1 exit)
   constexpr int n = R1 * R2, H = R1 / 2 + 1, NT = rfft_threads<R1, R2, TX>(), NIT = NT / TX;
@@ -159,12 +169,17 @@ __global__ void __launch_bounds__(rfft_threads<R1, R2, TX>(), rfft_ctas<T, R1, R
     for (int r = 1; r < R2; ++r) o[r * H * TX] = mul(tw[r * k1], z[r]);
   }
   __syncthreads();
-  // the scale 2^-log2(n) 2^-mex by exponent arithmetic in binary64 (one FP64 operation less)
-  int lg = 0;
-  while ((1 << lg) < n) ++lg;
-  const int ex = -lg - (mex && live ? mex[col / mnx] : 0);
-  const T inv_n = (T)ldexp(1.0, ex);
+  T inv_n = T(1) / T(n);
+  if (mex && live) inv_n = (T)ldexp((double)inv_n, -mex[col / mnx]);
   Tout *out = reinterpret_cast<Tout *>(outv) + col;
+  // batches: the store undoes the problem's scaling; columns that hold no unknown get exact zeros
+  int ex = 0;
+  bool dead = false;
+  if (SLOT && live) {
+    const int b = (int)(col / sc.mnx);
+    ex = -sc.ex[b];
+    dead = sc.zero[b] || col - (int64_t)b * sc.mnx >= sc.nxb[b];
+  }
   float ss = 0.0f;  // a few dozen squares per thread; the stop rule needs a few digits
   for (int r = it0; r < R2; r += NIT) {
     cpx<T> z[H];
@@ -184,16 +199,15 @@ __global__ void __launch_bounds__(rfft_threads<R1, R2, TX>(), rfft_ctas<T, R1, R
 #pragma unroll
       for (int i = 0; i < EB; ++i) {
         const int j = r + R2 * (i0 + i);
-        T v;
-        if constexpr (sizeof(T) == 8)
-          v = rsi ? x[i0 + i] * (inv_n * rsi[j]) : pow2_scale(x[i0 + i], ex);
-        else
-          v = x[i0 + i] * (rsi ? inv_n * rsi[j] : inv_n);
+        const T v = x[i0 + i] * (rsi ? inv_n * rsi[j] : inv_n);
         if (live) {
-          if constexpr (MODE == 1)
-            out[(int64_t)j * ldo] = old[i] + cvt<double>(v);
+          Tout d;
+          if constexpr (SLOT)
+            d = slot_store(v, ex);
           else
-            out[(int64_t)j * ldo] = cvt<Tout>(v);
+            d = cvt<Tout>(v);
+          if constexpr (MODE == 1) d = old[i] + d;
+          out[(int64_t)j * ldo] = SLOT && dead ? Tout(0) : d;
         }
         const float vf = cvt<float>(v);
         ss = fmaf(vf, vf, ss);
@@ -234,15 +248,18 @@ void rfft_tile(int n, int64_t ncols, F &&f) {
 
 template <typename T, typename Tin>
 void rfft_launch(Ctx &c, const Tin *X, int64_t ldx, int64_t ncols, int n, const cpx<T> *tw, cpx<T> *S, int64_t lds,
-                 const T *rs, const RhsNorm &rn, const char *fam, double bytes) {
+                 const T *rs, const RhsNorm &rn, const SlotScale &sc, const char *fam, double bytes) {
   c.launch(fam, bytes, [&] {
     rfft_tile<T>(n, ncols, [&](auto r1, auto r2, auto tx) {
       constexpr int R1 = decltype(r1)::value, R2 = decltype(r2)::value, TX = decltype(tx)::value;
       const size_t smem = (size_t)R2 * (R1 / 2 + 1) * TX * sizeof(cpx<T>);
-      auto kern = k_rfft<T, Tin, R1, R2, TX>;
+      auto kern = k_rfft<T, Tin, R1, R2, TX, false>;
+      if constexpr (sizeof(Tin) == 8) {
+        if (sc.ex) kern = k_rfft<T, Tin, R1, R2, TX, true>;
+      }
       if (smem > 48 * 1024) allow_dyn_smem((const void *)kern);
       pdl_launch(c.pdl, kern, dim3((unsigned)((ncols + TX - 1) / TX)), dim3(rfft_threads<R1, R2, TX>()), smem, c.stream,
-                 X, ldx, ncols, tw, S, lds, rs, rn);
+                 X, ldx, ncols, tw, S, lds, rs, rn, sc);
     });
   });
 }
@@ -250,20 +267,21 @@ void rfft_launch(Ctx &c, const Tin *X, int64_t ldx, int64_t ncols, int n, const 
 template <typename T>
 void crfft_launch(Ctx &c, const cpx<T> *S, int64_t lds, int64_t ncols, int n, const cpx<T> *tw, void *out, int64_t ldo,
                   int mode, double *norm_part, int *nparts, const StepFinish &fin, const T *rsi, double *colsum,
-                  const int *mex, int mnx, const int *skip, const char *fam, double bytes) {
+                  const int *mex, int mnx, const int *skip, const SlotScale &sc, const char *fam, double bytes) {
   c.launch(fam, bytes, [&] {
     rfft_tile<T>(n, ncols, [&](auto r1, auto r2, auto tx) {
       constexpr int R1 = decltype(r1)::value, R2 = decltype(r2)::value, TX = decltype(tx)::value;
       const size_t smem = (size_t)R2 * (R1 / 2 + 1) * TX * sizeof(cpx<T>);
-      auto kern = mode == 1 ? k_crfft<T, R1, R2, TX, 1> : k_crfft<T, R1, R2, TX, 0>;
+      auto kern = sc.ex ? (mode == 1 ? k_crfft<T, R1, R2, TX, 1, true> : k_crfft<T, R1, R2, TX, 0, true>)
+                        : (mode == 1 ? k_crfft<T, R1, R2, TX, 1, false> : k_crfft<T, R1, R2, TX, 0, false>);
       if constexpr (sizeof(T) == 4) {
-        if (mode == 2) kern = k_crfft<T, R1, R2, TX, 2>;
+        if (mode == 2) kern = k_crfft<T, R1, R2, TX, 2, false>;
       }
       if (smem > 48 * 1024) allow_dyn_smem((const void *)kern);
       const unsigned grid = (unsigned)((ncols + TX - 1) / TX);
       if (nparts) *nparts = (int)grid;
       pdl_launch(c.pdl, kern, dim3(grid), dim3(rfft_threads<R1, R2, TX>()), smem, c.stream, S, lds, ncols, tw, out, ldo,
-                 norm_part, fin, rsi, colsum, mex, mnx, skip);
+                 norm_part, fin, rsi, colsum, mex, mnx, skip, sc);
     });
   });
 }

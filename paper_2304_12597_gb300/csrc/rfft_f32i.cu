@@ -4,6 +4,6 @@
 namespace pd {
 
 template void crfft_launch<float>(Ctx &, const cpx<float> *, int64_t, int64_t, int, const cpx<float> *, void *, int64_t, int,
-    double *, int *, const StepFinish &, const float *, double *, const int *, int, const int *, const char *, double);
+    double *, int *, const StepFinish &, const float *, double *, const int *, int, const int *, const SlotScale &, const char *, double);
 
 }  // namespace pd
