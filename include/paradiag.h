@@ -300,8 +300,9 @@ pd_status paradiag_solve(pd_plan *plan, const double *G_dev, double *U_dev, pd_s
  * its solution; later calls keep refining it while it stays), 2 = it took max_refine + 1
  * solves without meeting it, 0 = still running (or an unused slot).
  * Each problem decides convergence by the same rules as in paradiag_solve, counted from
- * its own first solve.  The sweeps run as host-driven loops on the plan's stream; the call
- * returns after synchronising with it.  stats: this call's sweeps.
+ * its own first solve.  The sweeps run on the plan's stream, as host-driven loops or, from
+ * the eighth consecutive call with one (U_dev, steps) pair on, as one CUDA graph captured for that
+ * pair; the call returns after synchronising with the stream.  stats: this call's sweeps.
  * Errors: PD_ERR_INVALID_ARG (not a batched plan, steps outside [1, 64], NULL or aliasing
  * arguments), PD_ERR_UNSUPPORTED (fixed-loop variants, mass matrices), PD_ERR_NONFINITE. */
 pd_status paradiag_batch_advance(pd_plan *plan, const double *G_dev, double *U_dev, const int32_t *join,

@@ -291,9 +291,11 @@ struct pd_plan {
   const void *tail_src = nullptr;
   size_t tail_bytes = 0;
   bool tail_done = false;
+  bool ev1_done = false;  // the call's end event was recorded before its last synchronisation
   // pinned host mirrors of the scalar and flag blocks
   double *h_scal = nullptr;
-  int *h_flags = nullptr;
+  int *h_flags = nullptr;  // (in the same block as h_scal)
+  int *h_state = nullptr;  // (likewise: per-problem states of paradiag_batch_advance)
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   pd_stats last{};
   // CUDA graph of the whole solve, built for one (G, U) pair
@@ -303,9 +305,13 @@ struct pd_plan {
   cudaGraphExec_t gexec = nullptr;
   const double *g_G = nullptr;
   double *g_U = nullptr;
-  struct {
+  // CUDA graph of paradiag_batch_advance's sweeps, built for one (U, steps) pair
+  cudaGraphExec_t aexec = nullptr;
+  double *a_U = nullptr;
+  int a_steps = 0, a_calls = 0;  // a_calls: consecutive calls with this pair
+  struct Segments {
     int64_t pre0 = 0, iter0 = 0, post0 = 0, pre1 = 0, iter1 = 0, post1 = 0;
-  } seg;  // kernel launches per segment (for the launch count of graph solves)
+  } seg, aseg;  // kernel launches per segment (for the launch count of graph solves; aseg: of aexec)
 };
 
 namespace {
@@ -999,12 +1005,19 @@ pd_status ctx_status(pd_plan *p) {
   return PD_OK;
 }
 
-pd_status sync_read(pd_plan *p, bool with_tail = false) {
-  CK(cudaMemcpyAsync(p->h_scal, p->scal, pd::kScalWords * sizeof(double), cudaMemcpyDeviceToHost, p->ctx.stream));
-  CK(cudaMemcpyAsync(p->h_flags, p->flags, pd::kFlagWords * sizeof(int), cudaMemcpyDeviceToHost, p->ctx.stream));
-  if (with_tail && p->tail_dst) {
-    CK(cudaMemcpyAsync(p->tail_dst, p->tail_src, p->tail_bytes, cudaMemcpyDeviceToHost, p->ctx.stream));
-    p->tail_done = true;
+// Read the control block back (scal and flags are adjacent, here and there).  last: nothing of the
+// call follows, so its tail copy and its end event go in before the one synchronisation.
+constexpr size_t kControlBytes = pd::kScalWords * sizeof(double) + pd::kFlagWords * sizeof(int);
+static_assert(pd::kScalWords * sizeof(double) % 256 == 0, "flags follow scal in the workspace without a gap");
+pd_status sync_read(pd_plan *p, bool last = false) {
+  CK(cudaMemcpyAsync(p->h_scal, p->scal, kControlBytes, cudaMemcpyDeviceToHost, p->ctx.stream));
+  if (last) {
+    if (p->tail_dst) {
+      CK(cudaMemcpyAsync(p->tail_dst, p->tail_src, p->tail_bytes, cudaMemcpyDeviceToHost, p->ctx.stream));
+      p->tail_done = true;
+    }
+    CK(cudaEventRecord(p->ev1, p->ctx.stream));
+    p->ev1_done = true;
   }
   CK(cudaStreamSynchronize(p->ctx.stream));
   return ctx_status(p);
@@ -1498,7 +1511,7 @@ pd_status solve_hostloop(pd_plan *p, const double *G, double *U) {
 // Refinement sweeps only, on the U given (paradiag_batch_advance): the same kernels as the
 // host-driven loop, every solve a sweep on the FP64 residual, until the decision stops.
 template <typename T>
-pd_status solve_continue(pd_plan *p, const double *G, double *U) {
+pd_status continue_hostloop(pd_plan *p, const double *G, double *U) {
   pd::Ctx &c = p->ctx;
   pd_status st;
   pd::launch_solve_reset(c, p->scal, p->flags);
@@ -1562,9 +1575,39 @@ cudaError_t capture_iter_body(pd_plan *p, cudaGraph_t body, cudaStream_t s, int 
   return e;
 }
 
+// WHILE_R { pre(1), WHILE_k1 { iter(1) }, post(1) } after the capture frontier of cap[0].
 template <typename T>
-cudaError_t build_graph(pd_plan *p, const double *G, double *U, cudaGraph_t *gout) {
+cudaError_t capture_refine_loop(pd_plan *p, cudaGraphConditionalHandle hR, const double *G, double *U) {
   cudaStream_t s0 = p->cap[0], s1 = p->cap[1], s2 = p->cap[2];
+  cudaGraph_t bodyR = nullptr;
+  GK(splice_while(s0, hR, &bodyR));
+  cudaGraphConditionalHandle hk1;
+  GK(cudaGraphConditionalHandleCreate(&hk1, bodyR, 1, cudaGraphCondAssignDefault));
+  // refinement body: pre(1), WHILE_k1 { iter(1) }, post(1), captured on s1
+  GK(cudaStreamBeginCaptureToGraph(s1, bodyR, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed));
+  p->ctx.stream = s1;
+  int64_t l0 = p->ctx.launches;
+  bool ok = emit_pre<T>(p, 1, G, U, 1, hk1) == PD_OK;
+  p->seg.pre1 = p->ctx.launches - l0;
+  cudaGraph_t body1 = nullptr;
+  if (ok) ok = splice_while(s1, hk1, &body1) == cudaSuccess;
+  l0 = p->ctx.launches;
+  if (ok) ok = capture_iter_body<T>(p, body1, s2, 1, hk1) == cudaSuccess;
+  p->seg.iter1 = p->ctx.launches - l0;
+  p->ctx.stream = s1;
+  l0 = p->ctx.launches;
+  if (ok) ok = emit_post<T>(p, 1, U, 1, hR) == PD_OK;
+  p->seg.post1 = p->ctx.launches - l0;
+  cudaGraph_t outR = nullptr;
+  const cudaError_t e1 = cudaStreamEndCapture(s1, &outR);
+  return !ok || e1 != cudaSuccess || p->ctx.err != cudaSuccess ? cudaErrorUnknown : cudaSuccess;
+}
+
+// first = false: the refinement sweeps alone (paradiag_batch_advance), the first of them
+// unconditionally.
+template <typename T>
+cudaError_t build_graph(pd_plan *p, const double *G, double *U, cudaGraph_t *gout, bool first = true) {
+  cudaStream_t s0 = p->cap[0], s1 = p->cap[1];
   cudaStream_t keep = p->ctx.stream;
   cudaGraph_t g = nullptr;
   GK(cudaStreamBeginCapture(s0, cudaStreamCaptureModeRelaxed));
@@ -1572,12 +1615,17 @@ cudaError_t build_graph(pd_plan *p, const double *G, double *U, cudaGraph_t *gou
   do {
     cudaStreamCaptureStatus cs;
     if ((err = cudaStreamGetCaptureInfo(s0, &cs, nullptr, &g, nullptr, nullptr, nullptr)) != cudaSuccess) break;
-    cudaGraphConditionalHandle hk0, hR, hk1;
-    if ((err = cudaGraphConditionalHandleCreate(&hk0, g, 1, cudaGraphCondAssignDefault)) != cudaSuccess) break;
-    if ((err = cudaGraphConditionalHandleCreate(&hR, g, 0, cudaGraphCondAssignDefault)) != cudaSuccess) break;
+    cudaGraphConditionalHandle hk0, hR;
+    if ((err = cudaGraphConditionalHandleCreate(&hR, g, first ? 0 : 1, cudaGraphCondAssignDefault)) != cudaSuccess) break;
     p->ctx.stream = s0;
     int64_t l0 = p->ctx.launches;
     pd::launch_solve_reset(p->ctx, p->scal, p->flags);
+    if (!first) {
+      p->seg.pre0 = p->ctx.launches - l0;
+      err = capture_refine_loop<T>(p, hR, G, U);
+      break;
+    }
+    if ((err = cudaGraphConditionalHandleCreate(&hk0, g, 1, cudaGraphCondAssignDefault)) != cudaSuccess) break;
     if (emit_pre<T>(p, 0, G, U, 1, hk0) != PD_OK) { err = cudaErrorUnknown; break; }
     p->seg.pre0 = p->ctx.launches - l0;
     cudaGraph_t body = nullptr;
@@ -1589,32 +1637,7 @@ cudaError_t build_graph(pd_plan *p, const double *G, double *U, cudaGraph_t *gou
     l0 = p->ctx.launches;
     if (emit_post<T>(p, 0, U, 1, hR) != PD_OK) { err = cudaErrorUnknown; break; }
     p->seg.post0 = p->ctx.launches - l0;
-    cudaGraph_t bodyR = nullptr;
-    if ((err = splice_while(s0, hR, &bodyR)) != cudaSuccess) break;
-    if ((err = cudaGraphConditionalHandleCreate(&hk1, bodyR, 1, cudaGraphCondAssignDefault)) != cudaSuccess) break;
-    // refinement body: pre(1), WHILE_k1 { iter(1) }, post(1), captured on s1
-    if ((err = cudaStreamBeginCaptureToGraph(s1, bodyR, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed)) !=
-        cudaSuccess)
-      break;
-    p->ctx.stream = s1;
-    l0 = p->ctx.launches;
-    bool ok = emit_pre<T>(p, 1, G, U, 1, hk1) == PD_OK;
-    p->seg.pre1 = p->ctx.launches - l0;
-    cudaGraph_t body1 = nullptr;
-    if (ok) ok = splice_while(s1, hk1, &body1) == cudaSuccess;
-    l0 = p->ctx.launches;
-    if (ok) ok = capture_iter_body<T>(p, body1, s2, 1, hk1) == cudaSuccess;
-    p->seg.iter1 = p->ctx.launches - l0;
-    p->ctx.stream = s1;
-    l0 = p->ctx.launches;
-    if (ok) ok = emit_post<T>(p, 1, U, 1, hR) == PD_OK;
-    p->seg.post1 = p->ctx.launches - l0;
-    cudaGraph_t outR = nullptr;
-    const cudaError_t e1 = cudaStreamEndCapture(s1, &outR);
-    if (!ok || e1 != cudaSuccess || p->ctx.err != cudaSuccess) {
-      err = cudaErrorUnknown;
-      break;
-    }
+    if ((err = capture_refine_loop<T>(p, hR, G, U)) != cudaSuccess) break;
   } while (false);
   p->ctx.stream = keep;
   cudaGraph_t out = nullptr;
@@ -1628,11 +1651,67 @@ cudaError_t build_graph(pd_plan *p, const double *G, double *U, cudaGraph_t *gou
   return cudaSuccess;
 }
 
-void drop_graph(pd_plan *p) {
+void drop_solve_graph(pd_plan *p) {
   if (p->gexec) cudaGraphExecDestroy(p->gexec);
   p->gexec = nullptr;
   p->g_G = nullptr;
   p->g_U = nullptr;
+}
+
+void drop_advance_graph(pd_plan *p) {
+  if (p->aexec) cudaGraphExecDestroy(p->aexec);
+  p->aexec = nullptr;
+}
+
+void drop_graph(pd_plan *p) {
+  drop_solve_graph(p);
+  drop_advance_graph(p);
+}
+
+// The sweeps of one paradiag_batch_advance call (p->max_refine + 1 of them at most) as one graph
+// launch: the host synchronises once per call, not once per Algorithm-2 step and sweep (8 problems
+// of 2048 x 256 until all have converged, 4 calls: 1300 -> 1205 us; 8 of 63 x 63 x 128: 1320 -> 1227).
+// Capturing costs about as much as 30 calls gain, so a pair is captured at its kAdvanceCapture-th
+// consecutive call: a caller that brings a new U for each batch (a handful of calls) stays on the
+// host-driven loop and pays for no capture.
+constexpr int kAdvanceCapture = 8;
+template <typename T>
+pd_status solve_continue(pd_plan *p, double *U) {
+  if (!p->use_graphs || p->graph_failed || p->ctx.timing) return continue_hostloop<T>(p, nullptr, U);
+  if (p->a_U != U || p->a_steps != p->max_refine) {
+    drop_advance_graph(p);
+    p->a_U = U;
+    p->a_steps = p->max_refine;
+    p->a_calls = 0;
+  }
+  if (!p->aexec && ++p->a_calls < kAdvanceCapture) return continue_hostloop<T>(p, nullptr, U);
+  if (!p->aexec) {
+    std::lock_guard<std::recursive_mutex> lk(host_mutex());  // one capture at a time in the process
+    const int64_t l0 = p->ctx.launches;
+    const auto keep = p->seg;
+    cudaGraph_t g = nullptr;
+    cudaError_t e = build_graph<T>(p, nullptr, U, &g, false);
+    p->ctx.launches = l0;  // capture launches nothing
+    p->aseg = p->seg;
+    p->seg = keep;
+    if (e == cudaSuccess) e = cudaGraphInstantiate(&p->aexec, g, 0);
+    if (g) cudaGraphDestroy(g);
+    if (e != cudaSuccess || p->ctx.err != cudaSuccess) {
+      cudaGetLastError();
+      p->ctx.err = cudaSuccess;
+      p->aexec = nullptr;
+      p->graph_failed = true;
+      return continue_hostloop<T>(p, nullptr, U);
+    }
+  }
+  CK(cudaGraphLaunch(p->aexec, p->ctx.stream));
+  pd_status st = sync_read(p, true);
+  if (st != PD_OK) return st;
+  int64_t n = p->aseg.pre0;
+  for (int s = 0; s < p->h_flags[pd::F_SWEEP] && s < 16; ++s)
+    n += p->aseg.pre1 + p->aseg.post1 + (int64_t)p->aseg.iter1 * p->h_flags[pd::F_SWM + s];
+  p->ctx.launches += n;
+  return ctx_status(p);
 }
 
 template <typename T>
@@ -1641,7 +1720,7 @@ pd_status solve_graph(pd_plan *p, const double *G, double *U, bool *used) {
   if (p->graph_failed || p->ctx.timing) return PD_OK;
   if (!p->gexec || p->g_G != G || p->g_U != U) {
     std::lock_guard<std::recursive_mutex> lk(host_mutex());  // one capture at a time in the process
-    drop_graph(p);
+    drop_solve_graph(p);
     const int64_t l0 = p->ctx.launches;
     cudaGraph_t g = nullptr;
     cudaError_t e = build_graph<T>(p, G, U, &g);
@@ -1783,11 +1862,12 @@ pd_status paradiag_plan(const pd_desc *desc, void *workspace, size_t workspace_b
     paradiag_destroy(p);
     return s;
   };
-  if (cudaMallocHost(&p->h_scal, pd::kScalWords * sizeof(double)) != cudaSuccess ||
-      cudaMallocHost(&p->h_flags, pd::kFlagWords * sizeof(int)) != cudaSuccess)
+  // the control block's host side, and the states of paradiag_batch_advance
+  if (cudaMallocHost(&p->h_scal, kControlBytes + sizeof(int) * p->batch) != cudaSuccess)
     return cleanup(fail(PD_ERR_OOM, "cudaMallocHost failed"));
-  std::memset(p->h_scal, 0, pd::kScalWords * sizeof(double));
-  std::memset(p->h_flags, 0, pd::kFlagWords * sizeof(int));
+  p->h_flags = reinterpret_cast<int *>(p->h_scal + pd::kScalWords);
+  p->h_state = p->h_flags + pd::kFlagWords;
+  std::memset(p->h_scal, 0, kControlBytes);
   for (int i = 0; i < 3; ++i)
     if (cudaStreamCreateWithFlags(&p->cap[i], cudaStreamNonBlocking) != cudaSuccess)
       return cleanup(fail(PD_ERR_CUDA, "cudaStreamCreateWithFlags failed"));
@@ -1854,6 +1934,14 @@ pd_status paradiag_plan(const pd_desc *desc, void *workspace, size_t workspace_b
   if ((st = factorize(p)) != PD_OK) return cleanup(st);
   if (cudaMemsetAsync(p->flags, 0, pd::kFlagWords * sizeof(int), s) != cudaSuccess)
     return cleanup(fail(PD_ERR_CUDA, "plan upload failed"));
+  // paradiag_batch_advance on a problem that has never joined: its state reads as just joined
+  if (p->batch > 1 &&
+      (cudaMemsetAsync(p->mref2, 0, p->batch * sizeof(double), s) != cudaSuccess ||
+       cudaMemsetAsync(p->mprev, 0, p->batch * sizeof(double), s) != cudaSuccess ||
+       cudaMemsetAsync(p->mex, 0, p->batch * sizeof(int), s) != cudaSuccess ||
+       cudaMemsetAsync(p->msw, 0, p->batch * sizeof(int), s) != cudaSuccess ||
+       cudaMemsetAsync(p->mconv, 0, p->batch * sizeof(int), s) != cudaSuccess))
+    return cleanup(fail(PD_ERR_CUDA, "plan upload failed"));
   if (cudaStreamSynchronize(s) != cudaSuccess) return cleanup(fail(PD_ERR_CUDA, "plan upload failed"));
   *out = p;
   return PD_OK;
@@ -1895,7 +1983,6 @@ pd_status paradiag_destroy(pd_plan *p) {
   p->ctx.release();
   if (p->own_ws && p->ws) cudaFree(p->ws);
   if (p->h_scal) cudaFreeHost(p->h_scal);
-  if (p->h_flags) cudaFreeHost(p->h_flags);
   if (p->ev0) cudaEventDestroy(p->ev0);
   if (p->ev1) cudaEventDestroy(p->ev1);
   delete p;
@@ -1912,6 +1999,7 @@ pd_status paradiag_solve(pd_plan *p, const double *G, double *U, pd_stats *stats
   const char *g0 = reinterpret_cast<const char *>(G), *u0 = reinterpret_cast<const char *>(U);
   if (g0 < u0 + bytes && u0 < g0 + bytes) return fail(PD_ERR_INVALID_ARG, "U must not alias G");
   const int64_t l0 = p->ctx.launches;
+  p->ev1_done = false;
   CK(cudaEventRecord(p->ev0, p->ctx.stream));
   pd_stats s{};
   const double *Gin = G;
@@ -1927,8 +2015,10 @@ pd_status paradiag_solve(pd_plan *p, const double *G, double *U, pd_stats *stats
   st = p->precision == PD_FP64 ? solve_refined<double>(p, Gin, U, s) : solve_refined<float>(p, Gin, U, s);
   if (st == PD_ERR_CUDA) return st;
   if (p->mass) pd::launch_col_scale(p->ctx, U, U, p->nt, p->nbar, p->msc);  // u = M^{-1/2} w
-  CK(cudaEventRecord(p->ev1, p->ctx.stream));
-  CK(cudaEventSynchronize(p->ev1));
+  if (p->mass || !p->ev1_done) {
+    CK(cudaEventRecord(p->ev1, p->ctx.stream));
+    CK(cudaEventSynchronize(p->ev1));
+  }
   float ms = 0.f;
   cudaEventElapsedTime(&ms, p->ev0, p->ev1);
   s.ms_total = ms;
@@ -1955,6 +2045,7 @@ pd_status paradiag_batch_advance(pd_plan *p, const double *G, double *U, const i
   const char *g0 = reinterpret_cast<const char *>(G), *u0 = reinterpret_cast<const char *>(U);
   if (g0 < u0 + bytes && u0 < g0 + bytes) return fail(PD_ERR_INVALID_ARG, "U must not alias G");
   const int64_t l0 = p->ctx.launches;
+  p->ev1_done = false;
   CK(cudaEventRecord(p->ev0, p->ctx.stream));
   CK(cudaMemcpyAsync(p->mjoin, join, sizeof(int32_t) * p->batch, cudaMemcpyHostToDevice, p->ctx.stream));
   pd::launch_batch_exponents(p->ctx, G, p->nt, p->batch, (int)p->nxm, p->bnc, p->bpart, p->bex, p->bzero, p->gslot);
@@ -1963,15 +2054,27 @@ pd_status paradiag_batch_advance(pd_plan *p, const double *G, double *U, const i
   const int keep_max = p->max_refine;
   p->max_refine = steps - 1;         // this call's sweeps
   p->member_solves = keep_max + 1;   // each problem's own limit, counted over calls
-  st = p->precision == PD_FP64 ? solve_continue<double>(p, nullptr, U) : solve_continue<float>(p, nullptr, U);
+  p->tail_dst = p->h_state;
+  p->tail_src = p->mconv;
+  p->tail_bytes = sizeof(int) * p->batch;
+  p->tail_done = false;
+  st = p->precision == PD_FP64 ? solve_continue<double>(p, U) : solve_continue<float>(p, U);
   p->max_refine = keep_max;
   p->member_solves = 0;
+  const bool read = p->tail_done;
+  p->tail_dst = nullptr;
+  p->tail_src = nullptr;
+  p->tail_done = false;
   if (st == PD_ERR_CUDA) return st;
-  CK(cudaMemcpyAsync(state, p->mconv, sizeof(int32_t) * p->batch, cudaMemcpyDeviceToHost, p->ctx.stream));
-  CK(cudaEventRecord(p->ev1, p->ctx.stream));
-  CK(cudaEventSynchronize(p->ev1));
+  if (!read) {  // host-driven sweeps: the states and the end event still have to be read
+    CK(cudaMemcpyAsync(p->h_state, p->mconv, sizeof(int) * p->batch, cudaMemcpyDeviceToHost, p->ctx.stream));
+    CK(cudaEventRecord(p->ev1, p->ctx.stream));
+    CK(cudaEventSynchronize(p->ev1));
+  }
+  std::copy(p->h_state, p->h_state + p->batch, state);
   pd_stats s{};
   const int *f = p->h_flags;
+  s.graph = read ? 1 : 0;
   s.refine_sweeps = f[pd::F_SWEEP];
   s.krylov_iters_total = f[pd::F_MTOT];
   for (int i = 0; i < s.refine_sweeps && i < 16; ++i) {
