@@ -318,8 +318,8 @@ __global__ void __launch_bounds__(kFftMaxThreads) k_fft_r2c(const Tin *__restric
   if (rn.part) rhs_norm_finish((float)ss, rn);
 }
 
-// Same transform of the 1D FP64 residual r = G_t + u_{t-1} - (I + tau K) u_t, formed
-// while the tile is loaded (rx = (tau lo, 1 + tau diag, tau up)); neighbour columns
+// Same transform of the 1D FP64 residual r = G_t + u_{t-1} - (I + tau K) u_t (binary64, and binary32
+// outside the lengths of rfft_res.cu or with a tuned radix or tile), formed while the tile is loaded (rx = (tau lo, 1 + tau diag, tau up)); neighbour columns
 // outside the tile come from L1/L2.
 template <typename T, int TX, bool SLOT>
 __global__ void __launch_bounds__(kFftMaxThreads, 2) k_fft_r2c_res(const double *__restrict__ G, const double *__restrict__ U,
@@ -771,6 +771,10 @@ void launch_fft_r2c_residual(Ctx &c, const double *G, const double *U, int64_t n
   const size_t smem = (size_t)(TX / 2) * series_stride(n) * sizeof(cpx<T>);
   const int grid = (int)((ncols + TX - 1) / TX);
   const double bytes = (double)n * ncols * 16.0 + (double)(n / 2 + 1) * ncols * sizeof(cpx<T>);
+  if constexpr (sizeof(T) == 4) {
+    if (rfft_built<T>(c, n, ncols))
+      return rfft_res_launch<T>(c, G, U, ncols, n, rxl, rxd, rxu, tw, S, lds, rs, mex, mnx, rn, sc, "fft_r2c_res_f32", bytes);
+  }
   c.launch(sizeof(T) == 8 ? "fft_r2c_res_f64" : "fft_r2c_res_f32", bytes, [&] {
     PD_TX_DISPATCH(TX, {
       auto kern = sc.ex ? k_fft_r2c_res<T, kTX, true> : k_fft_r2c_res<T, kTX, false>;

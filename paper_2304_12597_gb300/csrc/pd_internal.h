@@ -213,6 +213,15 @@ template <typename T, typename Tin>
 void rfft_launch(Ctx &c, const Tin *X, int64_t ldx, int64_t ncols, int n, const cpx<T> *tw, cpx<T> *S, int64_t lds,
                  const T *rs, const RhsNorm &rn, const SlotScale &sc, const char *fam, double bytes);
 template <typename T>
+void rfft_res_launch(Ctx &c, const double *G, const double *U, int64_t ncols, int n, const double *rxl, const double *rxd,
+                     const double *rxu, const cpx<T> *tw, cpx<T> *S, int64_t lds, const T *rs, const int *mex, int mnx,
+                     const RhsNorm &rn, const SlotScale &sc, const char *fam, double bytes);
+template <>
+void rfft_res_launch<float>(Ctx &c, const double *G, const double *U, int64_t ncols, int n, const double *rxl,
+                            const double *rxd, const double *rxu, const cpx<float> *tw, cpx<float> *S, int64_t lds,
+                            const float *rs, const int *mex, int mnx, const RhsNorm &rn, const SlotScale &sc,
+                            const char *fam, double bytes);
+template <typename T>
 void crfft_launch(Ctx &c, const cpx<T> *S, int64_t lds, int64_t ncols, int n, const cpx<T> *tw, void *out, int64_t ldo,
                   int mode, double *norm_part, int *nparts, const StepFinish &fin, const T *rsi, double *colsum,
                   const int *mex, int mnx, const int *skip, const SlotScale &sc, const char *fam, double bytes);

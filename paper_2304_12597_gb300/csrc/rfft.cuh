@@ -18,8 +18,7 @@
 //    4095 columns of 2048, binary32   74 / 88 us -> 42 / 53 us,   binary64  411 / 418 us -> 347 / 371 us
 //   32736 columns of 1024, binary32  194 / 251 us -> 113 / 158 us
 //     300 columns of   32, binary32   14 / 15 us ->  8 / 12 us
-// The forward transform of the FP64 residual stays in fft.cu: it needs many loads in flight, and
-// measured 174 us here against 129 us there (4095 x 2048), with 64 rows a thread leaving too few warps.
+// The forward transform of the 1D FP64 residual, binary32, is in rfft_res.cu.
 #pragma once
 
 #include <algorithm>
@@ -55,6 +54,27 @@ constexpr int rfft_ctas() {
   constexpr int regs = R2 >= 32 || R1 >= 64 ? (sizeof(T) == 8 ? 168 : 112) : (sizeof(T) == 8 ? 112 : 72);
   constexpr int c = TX < wide_tx<T, R1, R2>() ? 2 : 65536 / (rfft_threads<R1, R2, TX>() * regs);
   return c < 1 ? 1 : c > 8 ? 8 : c;
+}
+
+// Forward, pass 2 for one k1: the frequencies k1 + R1 k2; past n/2 the conjugate of row n - k (rows 0
+// and R1/2 mod R1 hold their own mirror images).
+template <typename T, int R1, int R2, int TX>
+__device__ __forceinline__ void rfft_pass2(const cpx<T> *sm, cpx<T> *__restrict__ S, int64_t lds, int64_t col, bool live,
+                                           int k1) {
+  constexpr int n = R1 * R2, H = R1 / 2 + 1;
+  cpx<T> z[R2];
+  const cpx<T> *p = sm + k1 * TX;
+#pragma unroll
+  for (int r = 0; r < R2; ++r) z[r] = p[r * H * TX];
+  dft_reg<T, R2>(z);
+#pragma unroll
+  for (int k2 = 0; k2 < R2; ++k2) {
+    const int k = k1 + R1 * k2;
+    const bool up = 2 * k2 >= R2;
+    if (up && (k1 == H - 1 || (k1 == 0 && 2 * k2 > R2))) continue;
+    const bool mirror = up && k1 > 0;
+    if (live) S[(int64_t)(mirror ? n - k : k) * lds + col] = mirror ? conjg(z[k2]) : z[k2];
+  }
 }
 
 // Forward transform of X (n, ldx).
@@ -111,23 +131,7 @@ __global__ void __launch_bounds__(rfft_threads<R1, R2, TX>(), rfft_ctas<T, R1, R
     o[(H - 1) * TX] = scal(z[H - 1].x, tw[r * (H - 1)]);
   }
   __syncthreads();
-  for (int k1 = it0; k1 < H; k1 += NIT) {
-    cpx<T> z[R2];
-    const cpx<T> *p = sm + k1 * TX;
-#pragma unroll
-    for (int r = 0; r < R2; ++r) z[r] = p[r * H * TX];
-    dft_reg<T, R2>(z);
-    // frequencies k1 + R1 k2; past n/2 the conjugate of row n - k (rows 0 and R1/2 mod R1 hold their
-    // own mirror images)
-#pragma unroll
-    for (int k2 = 0; k2 < R2; ++k2) {
-      const int k = k1 + R1 * k2;
-      const bool up = 2 * k2 >= R2;
-      if (up && (k1 == H - 1 || (k1 == 0 && 2 * k2 > R2))) continue;
-      const bool mirror = up && k1 > 0;
-      if (live) S[(int64_t)(mirror ? n - k : k) * lds + col] = mirror ? conjg(z[k2]) : z[k2];
-    }
-  }
+  for (int k1 = it0; k1 < H; k1 += NIT) rfft_pass2<T, R1, R2, TX>(sm, S, lds, col, live, k1);
   if (rn.part) rhs_norm_finish(ss, rn);
 }
 
