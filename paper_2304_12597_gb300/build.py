@@ -15,7 +15,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OUT = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT, "libparadiag_gb300.so")
-SOURCES = ["fft.cu", "rfft_f32.cu", "rfft_f32i.cu", "rfft_res.cu", "rfft_f64.cu", "dst.cu", "pint.cu", "pint_chunk.cu", "krylov.cu", "krylov_members.cu", "control.cu", "plan.cu", "noalloc.cu", "batch.cu", "operator.cu"]
+SOURCES = ["fft.cu", "rfft_f32.cu", "rfft_f32i.cu", "rfft_res.cu", "rfft_f64.cu", "dst.cu", "pint.cu", "pint_chunk.cu", "pint_sys.cu", "krylov.cu", "krylov_members.cu", "control.cu", "plan.cu", "noalloc.cu", "batch.cu", "operator.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

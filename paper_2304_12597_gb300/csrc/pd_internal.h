@@ -296,6 +296,7 @@ struct PintGeom {
   int stage;     // 1: tau K staged in shared memory once per launch
   int chunk;     // 1: a geometry of k_pint_chunk (pint_chunk.cu): teams of P >= 8 lanes, a CTA per
                  // (block, split of the frequencies)
+  int sys;       // 1: a thread per (block, frequency) (pint_sys.cu, FP64)
 };
 // m_req / teams_req: rows per thread and teams per CTA requested by the caller (0 = choose);
 // fact: the loops will use stored factors (a smaller shared-memory footprint)
@@ -340,6 +341,7 @@ struct PintArgs {
   int xm_bpm;              // blocks per batch member (2D batches: the modes of its T_y; 0 = 1)
   const cpx<T> *fac_in;    // precomputed factors of every (k, block) system (pint.cu), or null
   cpx<T> *fac_out;         // factor pass: store those factors (R, rvec, Y, omega, V unused)
+  cpx<T> *scratch;         // pint_sys.cu: room for the forward sweep (pint_sys_scratch values)
   // Zero-frequency lane of the binary32 path.  A_0 = (1 - pi_0) I + tau K has the real
   // shift 1 - alpha^{1/l} (0 for Algorithm 1) and is the only ill-conditioned shifted
   // system (|1 - pi_k| >= 2 sin(pi / l) for k >= 1); its inverse (norm up to
@@ -362,6 +364,11 @@ size_t pint_factor_elems(const PintGeom &g);
 template <typename T>
 void launch_pint(Ctx &c, const PintGeom &g, const PintArgs<T> &a);
 void launch_pint_chunk(Ctx &c, const PintGeom &g, const PintArgs<float> &a);
+// FP64 loops with a thread per system (PintGeom::sys): they do not form the sums over the frequencies
+// (omega, acc_part), which the caller takes from the stored solutions.
+bool pint_sys_fits(int nf, int nblk);
+size_t pint_sys_scratch(const PintGeom &g);
+void launch_pint_sys(Ctx &c, const PintGeom &g, const PintArgs<double> &a);
 void launch_recip_f32(cudaStream_t s, const float *x, float *r, int64_t n);
 struct InitTail;  // pd_krylov.cuh: the start of Algorithm 2 run by a reduction's last CTA
 struct ProjTail;  // pd_krylov.cuh: eq. 13 and the step decision run by the z reduction's last CTA

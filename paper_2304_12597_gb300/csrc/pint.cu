@@ -83,6 +83,7 @@ __host__ __device__ inline int ilog2_pow2(int P) {
 __host__ __device__ inline int fac_slots(int M, int P) { return 4 * M - 4 + 2 * ilog2_pow2(P); }
 
 size_t pint_factor_elems(const PintGeom &g) {
+  if (g.sys) return 2 * pint_sys_scratch(g);
   return (size_t)g.nf * g.nblk * fac_slots(g.M, g.P) * g.P;
 }
 size_t pint_k0_factor_elems(const PintGeom &g) { return (size_t)g.nblk * fac_slots(g.M, g.P) * g.P; }
@@ -1061,6 +1062,8 @@ template <typename T>
 void launch_pint(Ctx &c, const PintGeom &g, const PintArgs<T> &a) {
   if constexpr (sizeof(T) == 4) {
     if (g.chunk) return launch_pint_chunk(c, g, a);
+  } else {
+    if (g.sys) return launch_pint_sys(c, g, a);
   }
   if (g.M == 4) {
     launch_pint_m<T, 4>(c, g, a);

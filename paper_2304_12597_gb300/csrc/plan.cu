@@ -227,6 +227,7 @@ struct pd_plan {
   double *msc = nullptr;  // M^{-1/2} (n_bar)
   double *Gm = nullptr;   // M^{-1/2} G (nt, n_bar)
   bool factored = false;  // the shifted systems are factored once per operator (fac)
+  cpx<double> *sysbuf = nullptr;  // PintArgs::scratch (geom.sys)
   void *fac = nullptr;
   double *mscal = nullptr;  // per-problem Algorithm-2 scalar and flag blocks
   int *mflags = nullptr;
@@ -608,6 +609,11 @@ void fill_geometry(pd_plan *p, const pd_desc *d) {
     const size_t esz = p->precision == PD_MIXED ? sizeof(cpx<float>) : sizeof(cpx<double>);
     const size_t fbytes = pd::pint_factor_elems(p->geom) * esz;
     p->factored = want_fac && fbytes <= ((size_t)4 << 30);
+    // FP64 plans with many systems give each a thread (pint_sys.cu), in less workspace than these
+    // factors take, unless the caller asked for factors, a launch geometry or the persistent step;
+    // vectors of one CTA keep the b reduction, whose last CTA starts Algorithm 2
+    p->geom.sys = p->factored && p->precision == PD_FP64 && !p->krylov_tails && d->tune_pint_factor == 0 &&
+                  !d->tune_pint_rows && !d->tune_pint_teams && d->tune_persistent <= 0 && pd::pint_sys_fits(p->nf, p->nblk);
   }
   p->ctx.pdl = d->tune_no_pdl == 0;
   // persistent Algorithm-2 step: single problems that run Algorithm 2.  The vector phases
@@ -703,6 +709,7 @@ size_t layout(pd_plan *p, unsigned char *base) {
   if (p->factored)
     p->fac = mixed ? (void *)A.take<cpx<float>>(pd::pint_factor_elems(p->geom))
                    : (void *)A.take<cpx<double>>(pd::pint_factor_elems(p->geom));
+  if (p->geom.sys) p->sysbuf = A.take<cpx<double>>(pd::pint_sys_scratch(p->geom));
   p->V = A.take<double>((size_t)(mx + 1) * nbar);
   if (mixed) {
     p->Vf = A.take<float>((size_t)(mx + 1) * nbar);
@@ -1067,6 +1074,7 @@ template <>
 pd::PintArgs<double> base_args<double>(pd_plan *p) {
   pd::PintArgs<double> a{};
   if (p->precision == PD_FP64) a.fac_in = reinterpret_cast<const cpx<double> *>(p->fac);
+  a.scratch = p->sysbuf;
   a.xm_scale = p->aroot;
   a.shift = p->shift;
   a.tlo = p->tlo_d;
@@ -1273,22 +1281,29 @@ pd_status emit_pre(pd_plan *p, int kind, const double *G, double *U, int use_han
   if constexpr (sizeof(T) == 4) a.omega_t = reinterpret_cast<const cpx<T> *>(p->wg_f);
   a.acc_part = p->acc_part;
   a.acc0 = lane_acc0<T>(p);
-  if (early || comb) {
+  const bool sys = loop_geom(p).sys;  // b from the stored L (the h_k buffer is free until Algorithm 2 starts)
+  if (early || comb || sys) {
     a.Y = L;
     a.ldy = p->lds;
   }
   pd::launch_pint<T>(c, loop_geom(p), a);
   pd::KrylovBufs kb = kbufs<T>(p);
   double *acc0 = lane_acc0<T>(p);
+  auto reduce_b = [&] {
+    if (sys)
+      pd::launch_zsum<T>(c, p->nf, p->nbar, L, p->lds, p->wg, p->b, nullptr);
+    else
+      pd::launch_acc_reduce(c, loop_geom(p), p->acc_part, p->b, nullptr, nullptr, acc0);
+  };
   if (kb.members) {
-    pd::launch_acc_reduce(c, loop_geom(p), p->acc_part, p->b, nullptr, nullptr, acc0);
+    reduce_b();
     pd::launch_member_init(c, kb, p->b, use_handle, hk);
   } else if (p->krylov_tails) {  // beta and v_1 in the b reduction's last CTA
     const pd::InitTail t{1, p->flags + pd::F_ACCCNT, kb.n, kb.maxit + 2, (kb.maxit + 1) * kb.maxit, use_handle,
                          kb.part, kb.V, kb.scal, kb.T, kb.Vf, kb.flags, hk};
     pd::launch_acc_reduce(c, loop_geom(p), p->acc_part, p->b, nullptr, &t, acc0);
   } else {
-    pd::launch_acc_reduce(c, loop_geom(p), p->acc_part, p->b, nullptr, nullptr, acc0);
+    reduce_b();
     pd::launch_vec_norm_init(c, kb, p->b, use_handle, hk);
   }
   // x_m = b: the inner matrix of eq. (17) taken as I (two loops in all)
@@ -2162,7 +2177,12 @@ pd_status paradiag_shifted_solve(pd_plan *p, const void *R, void *Y, double *b) 
       a.omega = p->wg;
       a.acc_part = p->acc_part;
     }
+    if (p->geom.sys && b && !Y) {  // b is summed from the stored solutions
+      a.Y = reinterpret_cast<cpx<double> *>(p->hbuf);
+      a.ldy = p->lds;
+    }
     pd::launch_pint<double>(p->ctx, p->geom, a);
+    if (p->geom.sys && b) pd::launch_zsum<double>(p->ctx, p->nf, p->nbar, a.Y, a.ldy, p->wg, b, nullptr);
   } else {
     pd::PintArgs<float> a = base_args<float>(p);
     a.k0_fp64 = 0;  // the stage entry point solves every frequency of arbitrary complex data in binary32
@@ -2176,7 +2196,7 @@ pd_status paradiag_shifted_solve(pd_plan *p, const void *R, void *Y, double *b) 
     }
     pd::launch_pint<float>(p->ctx, loop_geom(p), a);
   }
-  if (b) pd::launch_acc_reduce(p->ctx, loop_geom(p), p->acc_part, b, nullptr);
+  if (b && !loop_geom(p).sys) pd::launch_acc_reduce(p->ctx, loop_geom(p), p->acc_part, b, nullptr);
   CK(cudaStreamSynchronize(p->ctx.stream));
   return ctx_status(p);
 }
