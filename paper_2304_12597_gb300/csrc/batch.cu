@@ -12,14 +12,48 @@
 namespace pd {
 
 // part[b * nc + c] = sum over time rows t = c, c + nc, ... of slot b's squares.
+//
+// Only the exponent of the sum is used, so the squares are binary32, of values scaled by a power of two
+// taken from the largest of eight: integer work, one FP64 addition per eight values (an FP64 square of
+// each is 2 us per million on GB300's FP64 pipe, HBM 1.2 us).  Over- and underflow are those of binary64
+// squares.  W lanes (a power of two) share a row; eight loads are in flight per thread.  Measured with
+// the exponents kernel: 32 x 1023 x 1024 100 -> 77 us, 8 x 2048 x 256 33.6 -> 25 us.
+__device__ __forceinline__ double sumsq8(const double (&v)[8]) {
+  int e = 0;
+#pragma unroll
+  for (int u = 0; u < 8; ++u) e = max(e, (__double2hiint(v[u]) >> 20) & 0x7ff);
+  if (e == 0) return 0.0;  // zeros and subnormals, whose squares are zero
+  const int k = 1023 - e;
+  float s = 0.0f;
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    const float f = f64_to_f32_bits<true>(v[u], k);
+    s = fmaf(f, f, s);
+  }
+  return abs(k) <= 400 ? f32_to_f64_bits(s, -2 * k) : ldexp((double)s, -2 * k);
+}
 __global__ void __launch_bounds__(256) k_batch_sumsq(const double *__restrict__ X, int64_t nt, int64_t ld, int nxm,
-                                                     int nc, double *__restrict__ part) {
+                                                     int nc, double *__restrict__ part, int W) {
   grid_dep_wait();
   const int c = blockIdx.x, b = blockIdx.y;
+  const int i0 = (int)threadIdx.x & (W - 1);
+  const int64_t dt = (int64_t)nc * (256 / W);
+  const double *row = X + (int64_t)b * nxm;
   double s = 0.0;
-  for (int64_t t = c; t < nt; t += nc) {
-    const double *row = X + t * ld + (int64_t)b * nxm;
-    for (int i = threadIdx.x; i < nxm; i += blockDim.x) s = fma(row[i], row[i], s);
+  int64_t t = c + (int64_t)nc * (threadIdx.x / W);
+  int i = i0;
+  while (t < nt) {
+    double v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      v[u] = t < nt && i < nxm ? row[t * ld + i] : 0.0;
+      i += W;
+      if (i >= nxm) {
+        i = i0;
+        t += dt;
+      }
+    }
+    s += sumsq8(v);
   }
   __shared__ double red[8];
   s = warp_sum(s);
@@ -40,11 +74,13 @@ __global__ void __launch_bounds__(256) k_batch_sumsq(const double *__restrict__ 
 __global__ void k_batch_exponents(int batch, int nc, const double *__restrict__ part, int *__restrict__ ex,
                                   int *__restrict__ zero, const double *G, const double **gslot) {
   grid_dep_wait();
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b == 0) *gslot = G;
+  const int b = (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)), lane = threadIdx.x & 31;  // a warp per slot
+  if (blockIdx.x == 0 && threadIdx.x == 0) *gslot = G;
   if (b >= batch) return;
   double s = 0.0;
-  for (int c = 0; c < nc; ++c) s += part[(int64_t)b * nc + c];
+  for (int c = lane; c < nc; c += 32) s += part[(int64_t)b * nc + c];
+  s = warp_sum(s);
+  if (lane) return;
   int e = 0;
   if (s > 0.0 && isfinite(s)) {
     int e2;
@@ -58,11 +94,13 @@ __global__ void k_batch_exponents(int batch, int nc, const double *__restrict__ 
 void launch_batch_exponents(Ctx &c, const double *G, int64_t nt, int batch, int nxm, int nc, double *part, int *ex,
                             int *zero, const double **gslot) {
   const int64_t ld = (int64_t)batch * nxm;
+  int W = 32;
+  while (W < nxm && W < 256) W *= 2;
   c.launch("batch_scale", (double)nt * ld * 8.0, [&] {
-    pdl_launch(c.pdl, k_batch_sumsq, dim3(nc, batch), dim3(256), 0, c.stream, G, nt, ld, nxm, nc, part);
+    pdl_launch(c.pdl, k_batch_sumsq, dim3(nc, batch), dim3(256), 0, c.stream, G, nt, ld, nxm, nc, part, W);
   });
   c.launch("batch_scale", 0.0, [&] {
-    pdl_launch(c.pdl, k_batch_exponents, dim3((batch + 127) / 128), dim3(128), 0, c.stream, batch, nc, part, ex, zero, G,
+    pdl_launch(c.pdl, k_batch_exponents, dim3((batch + 7) / 8), dim3(256), 0, c.stream, batch, nc, part, ex, zero, G,
                gslot);
   });
 }
@@ -70,7 +108,7 @@ void launch_batch_exponents(Ctx &c, const double *G, int64_t nt, int batch, int 
 // A problem joining a running batch (join[b]): its U slot starts at zero and its refinement
 // state restarts; so does every unused slot (zero[b]: an all-zero right-hand side, whose U
 // may hold anything).  The other slots are not touched.
-__global__ void __launch_bounds__(256) k_member_join(double *U, int ld, int nxm, int batch, const int *__restrict__ join,
+__global__ void __launch_bounds__(256) k_member_join(double *U, int nt, int ld, int nxm, int batch, const int *__restrict__ join,
                                                      const int *__restrict__ zero, int *msw, double *prev, double *ref2,
                                                      int *mex, int *mconv) {
   grid_dep_wait();
@@ -84,15 +122,19 @@ __global__ void __launch_bounds__(256) k_member_join(double *U, int ld, int nxm,
   }
   if (j >= ld) return;
   const int b = j / nxm;
-  if (join[b] || zero[b]) U[(int64_t)blockIdx.y * ld + j] = 0.0;
+  if (join[b] || zero[b])
+    for (int t = blockIdx.y; t < nt; t += gridDim.y) U[(int64_t)t * ld + j] = 0.0;
 }
 
 void launch_member_join(Ctx &c, double *U, int64_t nt, int batch, int nxm, const int *join, const int *zero, int *msw,
                         double *prev, double *ref2, int *mex, int *mconv) {
   const int64_t ld = (int64_t)batch * nxm;
-  const dim3 grid((unsigned)((std::max<int64_t>(ld, batch) + 255) / 256), (unsigned)nt);
+  // enough CTAs to fill the SMs: most calls join few slots or none, and one CTA per row and 256
+  // columns spent its time on CTAs that had nothing to do (8 x 2048 x 256: 14.3 -> 7.2 us)
+  const unsigned gx = (unsigned)((std::max<int64_t>(ld, batch) + 255) / 256);
+  const dim3 grid(gx, (unsigned)std::min<int64_t>(nt, std::max<int64_t>(1, 8 * sm_count() / gx)));
   c.launch("batch_join", (double)nt * ld * 8.0, [&] {
-    pdl_launch(c.pdl, k_member_join, grid, dim3(256), 0, c.stream, U, (int)ld, nxm, batch, join, zero, msw, prev, ref2,
+    pdl_launch(c.pdl, k_member_join, grid, dim3(256), 0, c.stream, U, (int)nt, (int)ld, nxm, batch, join, zero, msw, prev, ref2,
                mex, mconv);
   });
 }
