@@ -784,8 +784,7 @@ __global__ void __launch_bounds__(kBlasSingle, 1) k_step_tail(StepArgs<T> a) {
 // cudaLaunchKernelEx (capturable into a CUDA graph).
 // Cluster variant: one CTA per SM (the dynamic shared memory request keeps a second
 // CTA off the SM), kBlasCluster threads each.
-constexpr int kClusterSpreadSmem = 120 * 1024;
-
+//
 // Largest cluster size <= want (halving, down to 4: with 128 threads per CTA and at most
 // 16 register-held entries per thread, 4 CTAs cover the 8192 entries one CTA would
 // take) the device can co-schedule for the cluster variant of the vector kernels; 0 if

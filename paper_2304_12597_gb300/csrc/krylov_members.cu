@@ -6,11 +6,13 @@
 // were solved alone.  The members share the kernel launches, the stored shifted
 // solves h_k and the basis array V (member b's entries in its own rows).
 //
-// One CTA per member holds that member's vectors in registers (len <= 8192 entries).
-// A member whose Algorithm 2 has stopped keeps its y_m and writes zero rows into V
-// from then on, so the shared shifted solves return zero there and x_m = V y_m stays
-// each member's own; the step loop runs while any member runs.  The last member to
-// finish the start or eq. (13) writes the batch totals and the loop decision.
+// A member's vectors are held in registers (len <= 8192 entries), by one thread-block cluster per
+// member while the clusters of all members fit the SMs, else by one CTA: a vector step is FP64 work,
+// and 512 threads on one SM per member left most SMs idle.  Measured per launch, init / Arnoldi /
+// eq. (13), one CTA -> clusters:
+//    8 members of 3969 rows  16.4 / 33.7 / 26.6 us -> 12.3 / 19.2 / 19.8 us (clusters of 8)
+//    8 members of 2048 rows  14.3 / 22.8 / 16.4 us -> 12.3 / 15.3 / 16.3 us (of 8)
+//   32 members of 1023 rows  14.3 / 16.8 / 16.3 us -> 12.2 / 15.3 / 18.3 us (of 4)
 #include "pd_internal.h"
 #include "pd_krylov.cuh"
 
@@ -80,32 +82,34 @@ __device__ void member_totals(const KrylovBufs &k, bool start, int use_handle, c
   }
 }
 
-// Start of Algorithm 2 for member blockIdx.x: beta_b = ||b_b||, v_1 = b_b / beta_b, its
+// Start of Algorithm 2 for member blockIdx.y: beta_b = ||b_b||, v_1 = b_b / beta_b, its
 // T_m and y_m cleared, its control block reset.
-template <int E>
-__global__ void __launch_bounds__(kBlasSingle) k_member_init(KrylovBufs k, const double *__restrict__ b,
+template <int MODE, int E>
+__global__ void __launch_bounds__(MODE == kCluster ? kBlasCluster : kBlasSingle) k_member_init(KrylovBufs k, const double *__restrict__ b,
                                                             int use_handle, cudaGraphConditionalHandle h) {
   grid_dep_wait();
   __shared__ double red[kRedWords];
   __shared__ double c[34];
-  const MemberView mv = member_view(k, blockIdx.x);
+  const MemberView mv = member_view(k, blockIdx.y);
   const int len = k.mlen;
-  for (int i = threadIdx.x; i < (k.maxit + 1) * k.maxit; i += blockDim.x) mv.T[i] = 0.0;
-  for (int i = threadIdx.x; i <= k.maxit; i += blockDim.x) mv.y[i] = 0.0;
+  __shared__ double cslot[MODE == kCluster ? kSlot : 1];
+  const int f = g_first<MODE>(), st = g_stride<MODE>();
+  for (int i = f; i < (k.maxit + 1) * k.maxit; i += st) mv.T[i] = 0.0;
+  for (int i = f; i <= k.maxit; i += st) mv.y[i] = 0.0;
   double x[E];
-  reg_load<kSingle, E>(len, b + mv.off, x);
-  const double beta = sqrt(reg_norm2<kSingle, E>(x, nullptr, 0, red, c));
+  reg_load<MODE, E>(len, b + mv.off, x);
+  const double beta = sqrt(reg_norm2<MODE, E>(x, cslot, 0, red, c));
   const double ib = beta > 0.0 ? 1.0 / beta : 0.0;
 #pragma unroll
   for (int e = 0; e < E; ++e) {
-    const int j = threadIdx.x + e * blockDim.x;
+    const int j = f + e * st;
     if (j < len) {
       const double v = x[e] * ib;
       k.V[mv.off + j] = v;
       if (k.Vf) k.Vf[mv.off + j] = (float)v;
     }
   }
-  if (threadIdx.x == 0) {
+  if (g_leader<MODE>()) {
     const bool finite = isfinite(beta), zero = !(beta > 0.0);
     double *scal = mv.scal;
     int *flags = mv.flags;
@@ -123,24 +127,26 @@ __global__ void __launch_bounds__(kBlasSingle) k_member_init(KrylovBufs k, const
     flags[F_KSTOP] = (finite && !zero) ? 0 : 1;
     flags[F_KCONV] = zero ? 1 : 0;
   }
+  cluster_exit<MODE>();
   if (last_cta_done(k.counter)) member_totals(k, true, use_handle, h, red);
 }
 
-// One Arnoldi step (eq. 10) for member blockIdx.x, as in the single-problem kernel;
+// One Arnoldi step (eq. 10) for member blockIdx.y, as in the single-problem kernel;
 // a member that has stopped writes a zero row instead.
-template <int E>
-__global__ void __launch_bounds__(kBlasSingle) k_member_arnoldi(KrylovBufs k) {
+template <int MODE, int E>
+__global__ void __launch_bounds__(MODE == kCluster ? kBlasCluster : kBlasSingle) k_member_arnoldi(KrylovBufs k) {
   grid_dep_wait();
   __shared__ double red[kRedWords];
   __shared__ double c[34];
-  const MemberView mv = member_view(k, blockIdx.x);
+  const MemberView mv = member_view(k, blockIdx.y);
   const int len = k.mlen, ldT = k.maxit;
   const int64_t ldv = k.n;
   const int m = k.flags[F_M] + 1;  // the step computed here produces row m of V
   double *vm = k.V + m * ldv + mv.off;
   float *vmf = k.Vf ? k.Vf + m * ldv + mv.off : nullptr;
-  if (mv.flags[F_KSTOP]) {
-    for (int j = threadIdx.x; j < len; j += blockDim.x) {
+  const int f = g_first<MODE>(), st = g_stride<MODE>();
+  if (mv.flags[F_KSTOP]) {  // uniform over the cluster
+    for (int j = f; j < len; j += st) {
       vm[j] = 0.0;
       if (vmf) vmf[j] = 0.0f;
     }
@@ -152,7 +158,7 @@ __global__ void __launch_bounds__(kBlasSingle) k_member_arnoldi(KrylovBufs k) {
   double x[E];
 #pragma unroll
   for (int e = 0; e < E; ++e) {
-    const int j = threadIdx.x + e * blockDim.x;
+    const int j = f + e * st;
     double a = 0.0;
     if (j < len) {
       a = kdiag[j] * v[j];
@@ -161,62 +167,68 @@ __global__ void __launch_bounds__(kBlasSingle) k_member_arnoldi(KrylovBufs k) {
     }
     x[e] = a;
   }
-  const bool wr = (int)threadIdx.x < m;  // writes column m-1 of T
-  reg_dots<kSingle, E>(len, m, Vb, ldv, x, nullptr, 0, red, c);
+  __shared__ double cslot[MODE == kCluster ? 3 * kSlot : 1];
+  double *const sl2 = MODE == kCluster ? cslot + kSlot : cslot, *const sl3 = MODE == kCluster ? cslot + 2 * kSlot : cslot;
+  const bool wr = (MODE == kSingle || blockIdx.x == 0) && (int)threadIdx.x < m;  // writes column m-1 of T
+  reg_dots<MODE, E>(len, m, Vb, ldv, x, cslot, 0, red, c);
   const double knorm = sqrt(c[m]);
   const double tq = wr ? c[threadIdx.x] : 0.0;
-  reg_axpy<kSingle, E>(len, m, Vb, ldv, x, c);
+  reg_axpy<MODE, E>(len, m, Vb, ldv, x, c);
   __syncthreads();  // c is rewritten next
-  reg_dots<kSingle, E>(len, m, Vb, ldv, x, nullptr, 0, red, c);
+  reg_dots<MODE, E>(len, m, Vb, ldv, x, sl2, 0, red, c);
   if (wr) mv.T[(int64_t)threadIdx.x * ldT + (m - 1)] = tq + c[threadIdx.x];
-  reg_axpy<kSingle, E>(len, m, Vb, ldv, x, c);
+  reg_axpy<MODE, E>(len, m, Vb, ldv, x, c);
   __syncthreads();
-  const double t = sqrt(cgs2_norm2<kSingle, E>(m, x, c, nullptr, 0, red));
+  const double t = sqrt(cgs2_norm2<MODE, E>(m, x, c, sl3, 0, red));
   const bool bd = !(t > 1e-14 * knorm);
   const double it = bd ? 0.0 : 1.0 / t;
 #pragma unroll
   for (int e = 0; e < E; ++e) {
-    const int j = threadIdx.x + e * blockDim.x;
+    const int j = f + e * st;
     if (j < len) {
       const double y = x[e] * it;
       vm[j] = y;
       if (vmf) vmf[j] = (float)y;
     }
   }
-  if (threadIdx.x == 0) {
+  if (g_leader<MODE>()) {
     mv.T[(int64_t)m * ldT + (m - 1)] = bd ? 0.0 : t;
     mv.scal[S_T] = bd ? 0.0 : t;
     mv.scal[S_KNORM] = knorm;
     mv.flags[F_BREAK] = bd ? 1 : 0;
     if (!isfinite(t)) mv.flags[F_NONFIN] = 1;
   }
+  cluster_exit<MODE>();
 }
 
-// eq. (13) for member blockIdx.x (two CGS passes of its part of z against its basis)
+// eq. (13) for member blockIdx.y (two CGS passes of its part of z against its basis)
 // and its stopping decision; members that had stopped keep their state.
-template <int E>
-__global__ void __launch_bounds__(kBlasSingle) k_member_project(KrylovBufs k, const double *__restrict__ z,
+template <int MODE, int E>
+__global__ void __launch_bounds__(MODE == kCluster ? kBlasCluster : kBlasSingle) k_member_project(KrylovBufs k, const double *__restrict__ z,
                                                                double tau, KrylovCtl kc, int use_handle,
                                                                cudaGraphConditionalHandle h) {
   grid_dep_wait();
   __shared__ double red[kRedWords];
   __shared__ double c[34];
-  const MemberView mv = member_view(k, blockIdx.x);
+  const MemberView mv = member_view(k, blockIdx.y);
   const int len = k.mlen;
   const int64_t ldv = k.n;
-  if (!mv.flags[F_KSTOP]) {  // the same for every thread of the CTA
+  if (!mv.flags[F_KSTOP]) {  // the same for every thread of the CTA and the cluster
+    __shared__ double cslot[MODE == kCluster ? 3 * kSlot : 1];
+    double *const sl2 = MODE == kCluster ? cslot + kSlot : cslot, *const sl3 = MODE == kCluster ? cslot + 2 * kSlot : cslot;
     const int m = mv.flags[F_M] + 1;
     const double *Vb = k.V + mv.off;
     double x[E];
-    reg_load<kSingle, E>(len, z + mv.off, x);
-    reg_dots<kSingle, E>(len, m, Vb, ldv, x, nullptr, 0, red, c);
-    reg_axpy<kSingle, E>(len, m, Vb, ldv, x, c);
+    reg_load<MODE, E>(len, z + mv.off, x);
+    reg_dots<MODE, E>(len, m, Vb, ldv, x, cslot, 0, red, c);
+    reg_axpy<MODE, E>(len, m, Vb, ldv, x, c);
     __syncthreads();  // c is rewritten next
-    reg_dots<kSingle, E>(len, m, Vb, ldv, x, nullptr, 0, red, c);
-    reg_axpy<kSingle, E>(len, m, Vb, ldv, x, c);
+    reg_dots<MODE, E>(len, m, Vb, ldv, x, sl2, 0, red, c);
+    reg_axpy<MODE, E>(len, m, Vb, ldv, x, c);
     __syncthreads();
-    const double zz = cgs2_norm2<kSingle, E>(m, x, c, nullptr, 0, red);
-    if (threadIdx.x == 0) {
+    const double zz = cgs2_norm2<MODE, E>(m, x, c, sl3, 0, red);
+    cluster_exit<MODE>();  // (before the decision changes the flags that the cluster's other CTAs read)
+    if (g_leader<MODE>()) {
       mv.scal[S_RES] = mv.flags[F_BREAK] ? 0.0 : fabs(tau * mv.scal[S_T]) * sqrt(zz);
       krylov_decide(mv.scal, mv.flags, kc, 0, h);
     }
@@ -224,37 +236,62 @@ __global__ void __launch_bounds__(kBlasSingle) k_member_project(KrylovBufs k, co
   if (last_cta_done(k.counter)) member_totals(k, false, use_handle, h, red);
 }
 
-static void member_launch(Ctx &c, const char *fam, double bytes, const void *fn, int members, void **args) {
+static void member_launch(Ctx &c, const char *fam, double bytes, const void *fn, const KrylovBufs &k, void **args) {
+  const int cl = k.cluster > 1 ? k.cluster : 1;
+  if (cl > 1) cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (cl > 1) allow_dyn_smem(fn);
   c.launch(fam, bytes, [&] {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)members);
-    cfg.blockDim = dim3(kBlasSingle);
+    cfg.gridDim = dim3((unsigned)cl, (unsigned)k.members);
+    cfg.blockDim = dim3(cl > 1 ? kBlasCluster : kBlasSingle);
+    cfg.dynamicSmemBytes = cl > 1 ? kClusterSpreadSmem : 0;
     cfg.stream = c.stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchAttribute attr[2];
+    int na = 0;
+    if (cl > 1) {
+      attr[na].id = cudaLaunchAttributeClusterDimension;
+      attr[na].val.clusterDim.x = (unsigned)cl;
+      attr[na].val.clusterDim.y = 1;
+      attr[na++].val.clusterDim.z = 1;
+    }
+    if (c.pdl) {
+      attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+      attr[na++].val.programmaticStreamSerializationAllowed = 1;
+    }
     cfg.attrs = attr;
-    cfg.numAttrs = c.pdl ? 1 : 0;
+    cfg.numAttrs = na;
     cudaLaunchKernelExC(&cfg, fn, args);
   });
 }
 
-#define PD_MEMBER_BY_E(E, KERNEL)                                                                    \
-  ((E) <= 1 ? (const void *)KERNEL<1>                                                               \
-            : (E) == 2 ? (const void *)KERNEL<2>                                                    \
-                       : (E) == 4 ? (const void *)KERNEL<4>                                         \
-                                  : (E) == 8 ? (const void *)KERNEL<8> : (const void *)KERNEL<16>)
+#define PD_MEMBER_E(E, KERNEL, MODE)                                                                 \
+  ((E) <= 1 ? (const void *)KERNEL<MODE, 1>                                                         \
+            : (E) == 2 ? (const void *)KERNEL<MODE, 2>                                              \
+                       : (E) == 4 ? (const void *)KERNEL<MODE, 4>                                   \
+                                  : (E) == 8 ? (const void *)KERNEL<MODE, 8> : (const void *)KERNEL<MODE, 16>)
+#define PD_MEMBER_BY_E(K, KERNEL)                                                                    \
+  ((K).cluster > 1 ? PD_MEMBER_E(reg_elems((K).mlen, (K).cluster * kBlasCluster), KERNEL, kCluster) \
+                   : PD_MEMBER_E(reg_elems((K).mlen, kBlasSingle), KERNEL, kSingle))
+
+// Clusters of 8 CTAs, of 4 while those of all members would not fit the SMs side by side; 0: one CTA
+// per member (more members than clusters of 4 leave room for, or short problems).  Eight clusters of 16
+// were slower than one CTA each (8 x 2048 rows: 16.3 / 21.8 / 22.4 us).
+int member_cluster_size(int members, int len) {
+  int want = 8;
+  while (want >= 4 && want * members > sm_count()) want >>= 1;
+  return want < 4 || len < 256 ? 0 : krylov_cluster_size(want);
+}
 
 void launch_member_init(Ctx &c, KrylovBufs &k, const double *b, int use_handle, cudaGraphConditionalHandle h) {
   void *args[] = {&k, (void *)&b, &use_handle, &h};
-  member_launch(c, "krylov_init", (double)k.n * 16, PD_MEMBER_BY_E(reg_elems(k.mlen, kBlasSingle), k_member_init),
-                k.members, args);
+  member_launch(c, "krylov_init", (double)k.n * 16, PD_MEMBER_BY_E(k, k_member_init),
+                k, args);
 }
 
 void launch_member_arnoldi(Ctx &c, KrylovBufs &k) {
   void *args[] = {&k};
   member_launch(c, "krylov_arnoldi", (double)k.n * 8.0 * 8,
-                PD_MEMBER_BY_E(reg_elems(k.mlen, kBlasSingle), k_member_arnoldi), k.members, args);
+                PD_MEMBER_BY_E(k, k_member_arnoldi), k, args);
 }
 
 void launch_member_project(Ctx &c, KrylovBufs &k, const double *z, double tau, const KrylovCtl &kc0, int use_handle,
@@ -262,7 +299,7 @@ void launch_member_project(Ctx &c, KrylovBufs &k, const double *z, double tau, c
   KrylovCtl kc = kc0;
   void *args[] = {&k, (void *)&z, &tau, &kc, &use_handle, &h};
   member_launch(c, "krylov_project", (double)k.n * 8.0 * 6,
-                PD_MEMBER_BY_E(reg_elems(k.mlen, kBlasSingle), k_member_project), k.members, args);
+                PD_MEMBER_BY_E(k, k_member_project), k, args);
 }
 
 }  // namespace pd

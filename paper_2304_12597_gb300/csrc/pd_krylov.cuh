@@ -26,6 +26,7 @@ namespace pd {
 
 constexpr int kBlasSingle = 512;   // threads of the one-CTA variants (short vectors)
 constexpr int kBlasCluster = 128;  // threads per CTA of the cluster variants
+constexpr int kClusterSpreadSmem = 120 * 1024;  // dynamic shared memory that keeps a cluster's CTAs on an SM each
 constexpr int kRedQ = 4;           // sums reduced side by side
 constexpr int kRedWords = kRedQ * kBlasSingle;
 constexpr int kSingle = 0, kCoop = 1, kCluster = 2, kTail = 3;  // MODE of the vector steps

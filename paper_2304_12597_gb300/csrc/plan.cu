@@ -591,6 +591,8 @@ void fill_geometry(pd_plan *p, const pd_desc *d) {
     p->blas_cluster = pd::krylov_cluster_size(want);
     if (p->blas_cluster < 4) p->blas_cluster = 0;
   }
+  if (p->members && d->tune_krylov_cluster >= 0)
+    p->blas_cluster = pd::member_cluster_size(p->members, (int)(p->nbar / p->members));
   // the start of Algorithm 2 and its eq. (13) decision are single-CTA work: with one CTA
   // they run in the last CTA of the reduction before them; with a cluster, on request
   p->krylov_tails = !p->members && p->blas_grid == 1 && d->tune_krylov_tails >= 0 &&
