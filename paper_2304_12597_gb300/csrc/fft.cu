@@ -10,6 +10,10 @@
 //   A[k] = (Z[k] + conj Z[-k]) / 2,   B[k] = (Z[k] - conj Z[-k]) / (2i).
 // Twiddles omega_n^k = exp(-2 pi i k / n), k < n/2, come from a table computed
 // on the host in FP64 (rounded to FP32 for the mixed path).
+//
+// The launchers below hand the lengths of the register transforms to them (rfft.cuh: n = 32 .. 2048;
+// dst.cu: n_y + 1 = 64, 128, 256); the kernels here take the other lengths, a caller's choice of
+// first-stage radix or tile, and the few shapes where those measured slower.
 #include <algorithm>
 
 #include "pd_control.cuh"

@@ -4,6 +4,11 @@
 // after the DST along y).  The ~l/2 systems are independent; pi_{l-k} =
 // conj(pi_k) makes the other half the complex conjugate.
 //
+// Binary32 loops without stored factors keep a chunk's rows in registers (pint_chunk.cu), and FP64
+// plans with many systems give each a thread (pint_sys.cu); this file's kernel takes the rest: FP64
+// plans of few systems, factored binary32 loops, the FP64 zero-frequency lane, and a caller's choice
+// of launch geometry.
+//
 // One team of P threads solves one tridiagonal block of `blen` rows:
 //  1. the right-hand side is staged in shared memory with coalesced loads;
 //  2. each thread eliminates its chunk of M rows so that every interior row

@@ -1688,8 +1688,8 @@ void drop_graph(pd_plan *p) {
 // The sweeps of one paradiag_batch_advance call (p->max_refine + 1 of them at most) as one graph
 // launch: the host synchronises once per call, not once per Algorithm-2 step and sweep (8 problems
 // of 2048 x 256 until all have converged, 4 calls: 1300 -> 1205 us; 8 of 63 x 63 x 128: 1320 -> 1227).
-// Capturing costs about as much as 30 calls gain, so a pair is captured at its kAdvanceCapture-th
-// consecutive call: a caller that brings a new U for each batch (a handful of calls) stays on the
+// Capturing costs some 0.1 ms, what four or five calls gain, so a pair is captured at its
+// kAdvanceCapture-th consecutive call: a caller that brings a new U for each batch (a handful of calls) stays on the
 // host-driven loop and pays for no capture.
 constexpr int kAdvanceCapture = 8;
 template <typename T>
