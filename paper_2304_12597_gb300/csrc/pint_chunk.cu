@@ -1,6 +1,6 @@
 // The binary32 parallel-in-time loop with chunks in registers: the shifted solves
 // ((1 - pi_k) I + tau K) y_k = r_k of pint.cu for plans that neither store factors nor run the
-// FP64 zero-frequency lane (those keep k_pint).
+// FP64 zero-frequency lane nor have rows far from diagonal dominance (those keep k_pint).
 //
 // One team of P lanes solves one tridiagonal block of blen <= P M rows; lane t owns the M
 // consecutive rows from t M in registers.
@@ -25,7 +25,10 @@
 // 1e-6 a sweep instead of 1e-3 to 1e-4, at about 25 % more arithmetic in this kernel (2D: 43 -> 44 us
 // per loop): advdiff1d_4095x2048 and heat2d_255x255x256 take 3 solves instead of 4 (1530 ->
 // 1160 us, 2964 -> 2234 us), 32 x heat1d_1023x1024 takes 3 instead of 5 (5336 -> 3297 us).
-// For other signs the same identities hold, with the rounding of a dominant elimination.
+// For other signs the same identities hold, with the rounding of the off-diagonals in place of the
+// diagonal's: harmless in rows that are dominant or nearly so, the only ones that come here
+// (suits_excess in plan.cu; a graded symmetric operator with off-diagonals 600 times the diagonal
+// left the refinement short of convergence).
 //
 // What bounds it: instruction issue.  Against k_pint's two separators per chunk of 8 rows held
 // in shared memory this takes 16 rows per lane (half the PCR levels per row), keeps aa, cc, r

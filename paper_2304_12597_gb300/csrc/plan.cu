@@ -232,7 +232,7 @@ struct pd_plan {
   double *mscal = nullptr;  // per-problem Algorithm-2 scalar and flag blocks
   int *mflags = nullptr;
   pd::PintGeom geom{};   // k_pint's teams
-  pd::PintGeom cgeom{};  // k_pint_chunk's teams (chunk = 0: not used by this plan)
+  pd::PintGeom cgeom{};  // k_pint_chunk's teams (chunk = 0: not used by this plan; see excess)
   int blas_grid = 1, k5_grid = 1;
   int k5_grid_members = 1;  // capacitance CTAs per problem of a batched plan
   int blas_cluster = 0;  // CTAs of the cluster variant of the one-CTA Krylov kernels (0 = off)
@@ -280,6 +280,7 @@ struct pd_plan {
   double *fac0 = nullptr;                 // PD_MIXED: the lane's FP64 factors (per operator)
   bool lane = false;                      // PD_MIXED: the zero frequency runs in the FP64 lane
   double nu0 = 0.0;                       // ||(l A_0)^{-1}||_inf estimate (lane criterion)
+  bool excess = false;                    // PD_MIXED: the operator's rows suit k_pint_chunk
   double2 *gpart = nullptr, *srow = nullptr, *omega = nullptr;
   double *msys_part = nullptr;
   double *norm_part = nullptr;
@@ -945,12 +946,38 @@ double zero_frequency_weight(const pd_plan *p, const HostOp &h) {
   return std::isfinite(worst) ? worst / (double)p->nt : 1e300;
 }
 
+// Whether the binary32 loops may eliminate from row sums (k_pint_chunk) instead of diagonals
+// (k_pint).  A pivot is then excess - (off-diagonals), whose rounding is that of the row's
+// off-diagonals: small against a dominant row's diagonal, but not against the diagonal of a
+// graded symmetric one (M^{-1/2} K M^{-1/2} with uneven masses, accepted as positive definite).
+// rho = (|lo| + |up|) / diag is at most 1 for dominant rows.  Measured as solves needed, k_pint_chunk /
+// k_pint (heat1d with random masses, n_x x n_t 300 x 64, 1023 x 256, 3000 x 64): rho 1.9 (masses within
+// a factor of 4): 3/3, 4/5, 4/6 (276/297, 414/518, 421/634 us); 3.6 (16): 3/3, 4/4, 5/5 (275/297,
+// 411/430, 507/542 us); 7 (64): 3/3, 4/4, 6/5 (275/296, 410/429, 597/542 us); 21 to 26 (1e3): 3/3, 5/4,
+// 9/5; 60 to 77 (1e4): 4/3, 6/4, 8/5; from 600 (1e6) on some do not converge with k_pint_chunk.
+constexpr double kExcessOff = 4.0;
+bool suits_excess(const pd_plan *p, const HostOp &h) {
+  for (int64_t i0 = 0; i0 < p->nrx; i0 += p->nxd) {  // the problems' T_x
+    double mu = 0.0;  // 2D: every block is T_x plus an eigenvalue of the problem's T_y
+    if (p->dim == 2) {
+      const auto m = h.mu.begin() + i0 / p->nxd * p->nym;
+      mu = *std::min_element(m, m + p->nym);
+    }
+    bool bad = false;
+    for (int64_t i = i0; i < i0 + p->nxd; ++i)
+      bad |= std::fabs(h.xlo[i]) + std::fabs(h.xup[i]) > kExcessOff * (h.xdiag[i] + mu);
+    if (bad) return false;
+  }
+  return true;
+}
+
 pd_status upload_operator(pd_plan *p, const pd_desc *desc) {
   pd_status st = PD_OK;
   const HostOp h = build_operator(desc);
   if (p->precision == PD_MIXED) {
     p->nu0 = zero_frequency_weight(p, h);
     p->lane = desc->tune_zero_lane > 0 || (desc->tune_zero_lane == 0 && p->nu0 > kLaneWeight);
+    p->excess = p->cgeom.chunk && suits_excess(p, h);
   }
   cudaStream_t s = p->ctx.stream;
   p->hop.clear();
@@ -1034,8 +1061,9 @@ pd_status sync_read(pd_plan *p, bool last = false) {
 
 // The final loop by linearity applies to single problems of the full method whose zero
 // frequency runs in binary32 like the others (the FP64 lane keeps the final loop's solves).
-// Geometry of the loops of an Algorithm-1 solve: the FP64 zero-frequency lane is k_pint's.
-const pd::PintGeom &loop_geom(const pd_plan *p) { return p->cgeom.chunk && !p->lane ? p->cgeom : p->geom; }
+// Geometry of the loops of an Algorithm-1 solve: the FP64 zero-frequency lane is k_pint's, and so are
+// operators whose row sums say too little about their pivots.
+const pd::PintGeom &loop_geom(const pd_plan *p) { return p->excess && !p->lane ? p->cgeom : p->geom; }
 
 bool use_comb(const pd_plan *p) { return p->comb && !(p->precision == PD_MIXED && p->lane); }
 
@@ -1982,9 +2010,10 @@ pd_status paradiag_set_operator(pd_plan *p, const pd_desc *desc) {
   }
   cudaStreamSynchronize(p->ctx.stream);  // no solve may still read the old operator, no upload its host side
   std::lock_guard<std::recursive_mutex> lk(host_mutex());
-  const bool lane_before = p->lane;
+  const bool lane_before = p->lane, excess_before = p->excess;
   if ((st = upload_operator(p, desc)) != PD_OK) return st;
-  if (p->lane != lane_before) drop_graph(p);  // the lane's arguments are captured in the graph
+  // the lane's arguments and the loops' kernel are captured in the graph
+  if (p->lane != lane_before || p->excess != excess_before) drop_graph(p);
   if ((st = factorize(p)) != PD_OK) return st;
   if (cudaStreamSynchronize(p->ctx.stream) != cudaSuccess) return fail(PD_ERR_CUDA, "operator upload failed");
   return PD_OK;
