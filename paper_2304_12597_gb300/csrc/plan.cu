@@ -337,11 +337,13 @@ struct HostOp {
 //      real part at least the corresponding pivot of the real LDL^T of tau K.
 // A diagonal mass matrix changes neither: (1 - pi_k) M + tau K is dominant when K is
 // (and has a positive definite Hermitian part when K is SPD), and the plan's symmetric
-// scaling M^{-1/2} (.) M^{-1/2} only rescales the rows and columns of its LU factors.
+// scaling M^{-1/2} (.) M^{-1/2} only rescales the rows and columns of its LU factors (it does not
+// keep row sums meaningful: suits_excess).
 // A centred advection term at cell Peclet number above 2 satisfies neither condition;
 // such operators are rejected rather than solved without pivoting.  The relative slack
 // 1e-12 absorbs the rounding of operators that are dominant with equality (upwind).
-pd_status check_dominance(const pd_desc *d) {
+pd_status check_dominance(const pd_desc *d, bool *all_dominant) {
+  if (all_dominant) *all_dominant = true;
   const int nb = d->batch > 1 ? d->batch : 1;
   for (int b = 0; b < nb; ++b) {
     double mu = 0.0;  // smallest eigenvalue of the problem's T_y (2D)
@@ -369,6 +371,7 @@ pd_status check_dominance(const pd_desc *d) {
       if (i + 1 < n && std::fabs(lo[i + 1] - u) > 1e-12 * (std::fabs(lo[i + 1]) + std::fabs(u))) symmetric = false;
     }
     if (dominant) continue;
+    if (all_dominant) *all_dominant = false;
     bool spd = symmetric;
     double h = 0.0;  // LDL^T pivots of the symmetric block
     for (int64_t i = 0; spd && i < n; ++i) {
@@ -385,7 +388,8 @@ pd_status check_dominance(const pd_desc *d) {
   return PD_OK;
 }
 
-pd_status validate(const pd_desc *d) {
+// dominant (optional): whether every row of K is diagonally dominant
+pd_status validate(const pd_desc *d, bool *dominant = nullptr) {
   if (!d) return fail(PD_ERR_INVALID_ARG, "desc is NULL");
   if (d->abi_version != PD_ABI_VERSION)
     return fail(PD_ERR_INVALID_ARG, "abi_version %d, library expects %d", d->abi_version, PD_ABI_VERSION);
@@ -499,7 +503,7 @@ pd_status validate(const pd_desc *d) {
   const int64_t nbar = d->nx * (d->dim == 2 ? d->ny : 1) * (d->batch > 1 ? d->batch : 1);
   if (nbar > (int64_t)1 << 28 || d->nt * nbar > (int64_t)1 << 34)
     return fail(PD_ERR_UNSUPPORTED, "problem too large for this build");
-  return check_dominance(d);
+  return check_dominance(d, dominant);
 }
 
 void fill_geometry(pd_plan *p, const pd_desc *d) {
@@ -950,7 +954,8 @@ double zero_frequency_weight(const pd_plan *p, const HostOp &h) {
 // (k_pint).  A pivot is then excess - (off-diagonals), whose rounding is that of the row's
 // off-diagonals: small against a dominant row's diagonal, but not against the diagonal of a
 // graded symmetric one (M^{-1/2} K M^{-1/2} with uneven masses, accepted as positive definite).
-// rho = (|lo| + |up|) / diag is at most 1 for dominant rows.  Measured as solves needed, k_pint_chunk /
+// rho = (|lo| + |up|) / diag is at most 1 for dominant rows, which validation has found already (looking
+// 16384 rows over again took 20 us of an operator swap).  Measured as solves needed, k_pint_chunk /
 // k_pint (heat1d with random masses, n_x x n_t 300 x 64, 1023 x 256, 3000 x 64): rho 1.9 (masses within
 // a factor of 4): 3/3, 4/5, 4/6 (276/297, 414/518, 421/634 us); 3.6 (16): 3/3, 4/4, 5/5 (275/297,
 // 411/430, 507/542 us); 7 (64): 3/3, 4/4, 6/5 (275/296, 410/429, 597/542 us); 21 to 26 (1e3): 3/3, 5/4,
@@ -971,13 +976,13 @@ bool suits_excess(const pd_plan *p, const HostOp &h) {
   return true;
 }
 
-pd_status upload_operator(pd_plan *p, const pd_desc *desc) {
+pd_status upload_operator(pd_plan *p, const pd_desc *desc, bool dominant) {
   pd_status st = PD_OK;
   const HostOp h = build_operator(desc);
   if (p->precision == PD_MIXED) {
     p->nu0 = zero_frequency_weight(p, h);
     p->lane = desc->tune_zero_lane > 0 || (desc->tune_zero_lane == 0 && p->nu0 > kLaneWeight);
-    p->excess = p->cgeom.chunk && suits_excess(p, h);
+    p->excess = p->cgeom.chunk && ((dominant && !desc->m_diag) || suits_excess(p, h));
   }
   cudaStream_t s = p->ctx.stream;
   p->hop.clear();
@@ -1878,7 +1883,8 @@ pd_status paradiag_workspace_size(const pd_desc *desc, size_t *bytes) {
 pd_status paradiag_plan(const pd_desc *desc, void *workspace, size_t workspace_bytes, pd_plan **out) {
   std::lock_guard<std::recursive_mutex> lk(host_mutex());
   g_err.clear();
-  pd_status st = validate(desc);
+  bool dominant = false;
+  pd_status st = validate(desc, &dominant);
   if (st != PD_OK) return st;
   if (!out) return fail(PD_ERR_INVALID_ARG, "out is NULL");
   *out = nullptr;
@@ -1975,7 +1981,7 @@ pd_status paradiag_plan(const pd_desc *desc, void *workspace, size_t workspace_b
     if ((st = upload(p->twy_d, ty.data(), N / 2, s)) || (st = upload(p->twy_f, tyf.data(), N / 2, s)))
       return cleanup(st);
   }
-  if ((st = upload_operator(p, desc)) != PD_OK) return cleanup(st);
+  if ((st = upload_operator(p, desc, dominant)) != PD_OK) return cleanup(st);
   if ((st = factorize(p)) != PD_OK) return cleanup(st);
   if (cudaMemsetAsync(p->flags, 0, pd::kFlagWords * sizeof(int), s) != cudaSuccess)
     return cleanup(fail(PD_ERR_CUDA, "plan upload failed"));
@@ -1995,7 +2001,8 @@ pd_status paradiag_plan(const pd_desc *desc, void *workspace, size_t workspace_b
 pd_status paradiag_set_operator(pd_plan *p, const pd_desc *desc) {
   pd_status st = check_plan(p);
   if (st != PD_OK) return st;
-  if ((st = validate(desc)) != PD_OK) return st;
+  bool dominant = false;
+  if ((st = validate(desc, &dominant)) != PD_OK) return st;
   const int batch = desc->batch > 1 ? desc->batch : 1;
   const int64_t ny = desc->dim == 2 ? desc->ny : 1;
   if (desc->dim != p->dim || desc->nx != p->nxd || ny != p->nym || desc->nt != p->nt || batch != p->batch ||
@@ -2011,7 +2018,7 @@ pd_status paradiag_set_operator(pd_plan *p, const pd_desc *desc) {
   cudaStreamSynchronize(p->ctx.stream);  // no solve may still read the old operator, no upload its host side
   std::lock_guard<std::recursive_mutex> lk(host_mutex());
   const bool lane_before = p->lane, excess_before = p->excess;
-  if ((st = upload_operator(p, desc)) != PD_OK) return st;
+  if ((st = upload_operator(p, desc, dominant)) != PD_OK) return st;
   // the lane's arguments and the loops' kernel are captured in the graph
   if (p->lane != lane_before || p->excess != excess_before) drop_graph(p);
   if ((st = factorize(p)) != PD_OK) return st;
