@@ -238,11 +238,11 @@ __global__ void __launch_bounds__(NW * 32, MINB)
         const T a = (upper ? -sa : sa) * v.y, b = (upper ? -sb : sb) * v.x;
         Tout da, db;
         if constexpr (SLOT && sizeof(Tout) == 8) {
-          da = slot_store(a, c[0].eout);
-          db = slot_store(b, c[1].eout);
+          da = slot_store<true>(a, c[0].eout);
+          db = slot_store<true>(b, c[1].eout);
         } else {
-          da = cvt<Tout>(a);
-          db = cvt<Tout>(b);
+          da = cvt<Tout, true>(a);
+          db = cvt<Tout, true>(b);
         }
         if (MODE == 1) {
           da = oa[u] + da;
