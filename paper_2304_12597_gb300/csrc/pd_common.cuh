@@ -150,21 +150,14 @@ __device__ __forceinline__ To cvt(From x) {
     return (To)x;
 }
 
-// x * 2^k by an exponent-field add (|k| < 1000): exact where the result is a normal number; below
-// that, zero; zero, infinities and NaN stay.  The batches' scale factors come from sums of squares
-// in binary64, so their exponents lie within +-540 and the rest of a problem far above that floor.
+// x * 2^k (|k| <= 1000) as ldexp gives it: an exponent-field add for a normal x whose result is normal; else
+// (zero, subnormal, infinity, NaN, under- or overflow) a multiplication by the power of two, exact or
+// rounded once.  8 x 63 x 63 x 128 in FP64 takes 3971 us; 4031 us with the multiplication for every value,
+// an FP64 operation each; 3920 us with flushed subnormals.
 __device__ __forceinline__ double pow2_scale(double x, int k) {
-  const int hi = __double2hiint(x), e = (hi >> 20) & 0x7ff, t = e + k;
-  int h = hi + (k << 20), l = __double2loint(x);
-  if (t >= 0x7ff) {  // overflow: infinity
-    h = (hi & 0x80000000) | 0x7ff00000;
-    l = 0;
-  }
-  if (e == 0 || t <= 0) {
-    h = hi & 0x80000000;
-    l = 0;
-  }
-  return e == 0x7ff ? x : __hiloint2double(h, l);
+  const int hi = __double2hiint(x), e = (hi >> 20) & 0x7ff;
+  if ((unsigned)(e - 1) < 0x7feu && (unsigned)(e + k - 1) < 0x7feu) return __hiloint2double(hi + (k << 20), __double2loint(x));
+  return x * __hiloint2double((1023 + k) << 20, 0);
 }
 // Problem scaling of the batches on load and store: x 2^k in type T, and back to binary64.
 template <typename T>
