@@ -11,27 +11,12 @@
 
 namespace pd {
 
-// part[b * nc + c] = sum over time rows t = c, c + nc, ... of slot b's squares.
+// part[b * nc + c] = sum over time rows t = c, c + nc, ... of slot b's squares, in binary64.
 //
-// Only the exponent of the sum is used, so the squares are binary32, of values scaled by a power of two
-// taken from the largest of eight: integer work, one FP64 addition per eight values (an FP64 square of
-// each is 2 us per million on GB300's FP64 pipe, HBM 1.2 us).  Over- and underflow are those of binary64
-// squares.  W lanes (a power of two) share a row; eight loads are in flight per thread.  Measured with
-// the exponents kernel: 32 x 1023 x 1024 100 -> 77 us, 8 x 2048 x 256 33.6 -> 25 us.
-__device__ __forceinline__ double sumsq8(const double (&v)[8]) {
-  int e = 0;
-#pragma unroll
-  for (int u = 0; u < 8; ++u) e = max(e, (__double2hiint(v[u]) >> 20) & 0x7ff);
-  if (e == 0) return 0.0;  // zeros and subnormals, whose squares are zero
-  const int k = 1023 - e;
-  float s = 0.0f;
-#pragma unroll
-  for (int u = 0; u < 8; ++u) {
-    const float f = f64_to_f32_bits<true>(v[u], k);
-    s = fmaf(f, f, s);
-  }
-  return abs(k) <= 400 ? f32_to_f64_bits(s, -2 * k) : ldexp((double)s, -2 * k);
-}
+// Bound by GB300's FP64 pipe (2 us per million squares; HBM 1.2).  W lanes (a power of two) share a row;
+// eight loads are in flight per thread, and the squares go into two chains.  Measured with the exponents
+// kernel, against one load at a time: 32 x 1023 x 1024 100 -> 83 us, 8 x 2048 x 256 33.6 -> 25.6 us.
+// (Binary32 squares took 77 and 25 us, and lost half of the digits.)
 __global__ void __launch_bounds__(256) k_batch_sumsq(const double *__restrict__ X, int64_t nt, int64_t ld, int nxm,
                                                      int nc, double *__restrict__ part, int W) {
   grid_dep_wait();
@@ -39,7 +24,7 @@ __global__ void __launch_bounds__(256) k_batch_sumsq(const double *__restrict__ 
   const int i0 = (int)threadIdx.x & (W - 1);
   const int64_t dt = (int64_t)nc * (256 / W);
   const double *row = X + (int64_t)b * nxm;
-  double s = 0.0;
+  double s0 = 0.0, s1 = 0.0;
   int64_t t = c + (int64_t)nc * (threadIdx.x / W);
   int i = i0;
   while (t < nt) {
@@ -53,10 +38,14 @@ __global__ void __launch_bounds__(256) k_batch_sumsq(const double *__restrict__ 
         t += dt;
       }
     }
-    s += sumsq8(v);
+#pragma unroll
+    for (int u = 0; u < 8; u += 2) {
+      s0 = fma(v[u], v[u], s0);
+      s1 = fma(v[u + 1], v[u + 1], s1);
+    }
   }
   __shared__ double red[8];
-  s = warp_sum(s);
+  const double s = warp_sum(s0 + s1);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
   __syncthreads();
   if (threadIdx.x == 0) {
