@@ -112,6 +112,10 @@ __device__ __forceinline__ float f64_to_f32_bits(double x, int k = 0) {
   }
   return __uint_as_float(r);
 }
+// The same rounded to nearest (ties away from zero); infinities become NaN.
+__device__ __forceinline__ float f64_to_f32_near(double x) {
+  return f64_to_f32_bits(__longlong_as_double(__double_as_longlong(x) + 0x10000000LL));
+}
 // binary32 -> binary64 by integer operations, for the same reason (the stores of the inverse
 // transforms: one conversion beside the one FP64 add of U += delta).  Exact for every finite number and
 // infinity; NaN stays NaN.  k: times 2^k, |k| <= 800 (every binary32 number then stays normal in

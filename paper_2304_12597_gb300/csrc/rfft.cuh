@@ -14,9 +14,10 @@
 // some 150 of the shared-memory passes in fft.cu); with the FP64 update on store, and in binary64,
 // GB300's FP64 pipe (about 20 operations per unknown, against 25).  Measured per launch (one GB300,
 // fft.cu -> here; forward / inverse):
-//   65025 columns of  256, binary32   56 / 85 us -> 42 / 46 us,   binary64  614 / 669 us -> 412 / 479 us
-//    4095 columns of 2048, binary32   74 / 88 us -> 42 / 53 us,   binary64  411 / 418 us -> 347 / 371 us
+//   65025 columns of  256, binary32   56 / 85 us -> 42 / 46 us,   binary64  614 / 669 us -> 435 / 480 us
+//    4095 columns of 2048, binary32   74 / 88 us -> 42 / 53 us,   binary64  411 / 418 us -> 350 / 371 us
 //   32736 columns of 1024, binary32  194 / 251 us -> 113 / 158 us
+//     (forward with the norm of the input, in binary64 one FP64 operation per value: 23 of the 435 us)
 //     300 columns of   32, binary32   14 / 15 us ->  8 / 12 us
 // The forward transform of the 1D FP64 residual, binary32, is in rfft_res.cu.
 #pragma once
@@ -89,7 +90,7 @@ __global__ void __launch_bounds__(rfft_threads<R1, R2, TX>(), rfft_ctas<T, R1, R
   cpx<T> *sm = reinterpret_cast<cpx<T> *>(smraw) + cl;  // (r, k1) at (r H + k1) TX
   const int64_t col = (int64_t)blockIdx.x * TX + cl;
   const bool live = col < ncols;
-  float ss = 0.0f;  // squares of the input (rn: a reference scale)
+  T ss = T(0);  // squares of the input (rn: a reference scale)
   int ex = 0;
   if constexpr (SLOT) {
     X = global_ptr(sc.G);
@@ -113,10 +114,7 @@ __global__ void __launch_bounds__(rfft_threads<R1, R2, TX>(), rfft_ctas<T, R1, R
     }
     if (rn.part) {
 #pragma unroll
-      for (int i = 0; i < R1; ++i) {
-        const float f = cvt<float>(x[i]);
-        ss = fmaf(f, f, ss);
-      }
+      for (int i = 0; i < R1; ++i) ss += x[i] * x[i];
     }
     if (rs) {
 #pragma unroll
@@ -132,7 +130,7 @@ __global__ void __launch_bounds__(rfft_threads<R1, R2, TX>(), rfft_ctas<T, R1, R
   }
   __syncthreads();
   for (int k1 = it0; k1 < H; k1 += NIT) rfft_pass2<T, R1, R2, TX>(sm, S, lds, col, live, k1);
-  if (rn.part) rhs_norm_finish(ss, rn);
+  if (rn.part) rhs_norm_finish((float)ss, rn);
 }
 
 // Inverse: X[j] = Re((1/n) sum_k w_n^{-jk} Y[k]) with Y[n - k] = conj Y[k], times rsi[j] and, for
@@ -213,7 +211,11 @@ __global__ void __launch_bounds__(rfft_threads<R1, R2, TX>(), rfft_ctas<T, R1, R
           if constexpr (MODE == 1) d = old[i] + d;
           out[(int64_t)j * ldo] = SLOT && dead ? Tout(0) : d;
         }
-        const float vf = cvt<float>(v);
+        float vf;
+        if constexpr (sizeof(T) == 8)
+          vf = f64_to_f32_near(v);
+        else
+          vf = v;
         ss = fmaf(vf, vf, ss);
       }
     }
