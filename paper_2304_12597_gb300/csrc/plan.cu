@@ -1757,10 +1757,8 @@ pd_status solve_continue(pd_plan *p, double *U) {
   CK(cudaGraphLaunch(p->aexec, p->ctx.stream));
   pd_status st = sync_read(p, true);
   if (st != PD_OK) return st;
-  int64_t n = p->aseg.pre0;
-  for (int s = 0; s < p->h_flags[pd::F_SWEEP] && s < 16; ++s)
-    n += p->aseg.pre1 + p->aseg.post1 + (int64_t)p->aseg.iter1 * p->h_flags[pd::F_SWM + s];
-  p->ctx.launches += n;
+  p->ctx.launches += p->aseg.pre0 + (int64_t)p->h_flags[pd::F_SWEEP] * (p->aseg.pre1 + p->aseg.post1) +
+                     (int64_t)p->h_flags[pd::F_MTOT] * p->aseg.iter1;
   return ctx_status(p);
 }
 
@@ -1792,11 +1790,10 @@ pd_status solve_graph(pd_plan *p, const double *G, double *U, bool *used) {
   pd_status st = sync_read(p, true);
   if (st != PD_OK) return st;
   // kernels run = fixed segments + m steps of Algorithm 2 per solve
-  const int sweeps = p->h_flags[pd::F_SWEEP];
-  int64_t n = p->seg.pre0 + p->seg.post0 + (int64_t)p->seg.iter0 * p->h_flags[pd::F_SWM];
-  for (int s = 1; s < sweeps && s < 16; ++s)
-    n += p->seg.pre1 + p->seg.post1 + (int64_t)p->seg.iter1 * p->h_flags[pd::F_SWM + s];
-  p->ctx.launches += n;
+  const int m0 = p->h_flags[pd::F_SWM];
+  p->ctx.launches += p->seg.pre0 + p->seg.post0 + (int64_t)m0 * p->seg.iter0 +
+                     (int64_t)std::max(0, p->h_flags[pd::F_SWEEP] - 1) * (p->seg.pre1 + p->seg.post1) +
+                     (int64_t)(p->h_flags[pd::F_MTOT] - m0) * p->seg.iter1;
   *used = true;
   return PD_OK;
 }
