@@ -149,7 +149,9 @@ typedef struct pd_desc {
   int32_t tune_krylov_cluster; /* where one CTA would run the Krylov vector kernels: -1 =
                                 keep that single CTA; 4 .. 16 = spread them over a
                                 thread-block cluster of that many CTAs, one per SM, with the
-                                reductions through distributed shared memory */
+                                reductions through distributed shared memory (batches: a
+                                cluster per problem; 0 = of 8 or 4 while those of all problems
+                                fit the SMs, else one CTA each) */
   int32_t tune_pint_factor;  /* 1: factor every shifted system once per operator (plan
                                 creation, paradiag_set_operator) and keep the factors (at
                                 most 4 GiB), so each parallel-in-time loop only solves; -1:

@@ -275,10 +275,13 @@ static void member_launch(Ctx &c, const char *fam, double bytes, const void *fn,
 
 // Clusters of 8 CTAs, of 4 while those of all members would not fit the SMs side by side; 0: one CTA
 // per member (more members than clusters of 4 leave room for, or short problems).  Eight clusters of 16
-// were slower than one CTA each (8 x 2048 rows: 16.3 / 21.8 / 22.4 us).
-int member_cluster_size(int members, int len) {
-  int want = 8;
-  while (want >= 4 && want * members > sm_count()) want >>= 1;
+// were slower than one CTA each (8 x 2048 rows: 16.3 / 21.8 / 22.4 us).  A caller's size (want > 0) is taken
+// as it is, as for single problems; clusters that do not fit side by side run one after another.
+int member_cluster_size(int members, int len, int want) {
+  if (want <= 0) {
+    want = 8;
+    while (want >= 4 && want * members > sm_count()) want >>= 1;
+  }
   return want < 4 || len < 256 ? 0 : krylov_cluster_size(want);
 }
 

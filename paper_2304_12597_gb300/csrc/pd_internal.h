@@ -434,7 +434,7 @@ void launch_arnoldi(Ctx &c, KrylovBufs &k);
 // Largest cluster size <= want (halving, >= 4) the device can co-schedule for the
 // cluster variant of the vector kernels (one CTA per SM); 0 if none.
 int krylov_cluster_size(int want);
-int member_cluster_size(int members, int len);  // the same for batched plans (krylov_members.cu)
+int member_cluster_size(int members, int len, int want);  // batched plans (krylov_members.cu); want 0: choose
 void launch_capacitance(Ctx &c, KrylovBufs &k, int nf, double tau, const double2 *shift,
                         const double2 *wg, const double2 *gpart, int nblk, double *msys_part,
                         int k5_grid, double2 *srow, double2 *omega, double *y, int members = 0, int bpm = 1,

@@ -597,7 +597,7 @@ void fill_geometry(pd_plan *p, const pd_desc *d) {
     if (p->blas_cluster < 4) p->blas_cluster = 0;
   }
   if (p->members && d->tune_krylov_cluster >= 0)
-    p->blas_cluster = pd::member_cluster_size(p->members, (int)(p->nbar / p->members));
+    p->blas_cluster = pd::member_cluster_size(p->members, (int)(p->nbar / p->members), d->tune_krylov_cluster);
   // the start of Algorithm 2 and its eq. (13) decision are single-CTA work: with one CTA
   // they run in the last CTA of the reduction before them; with a cluster, on request
   p->krylov_tails = !p->members && p->blas_grid == 1 && d->tune_krylov_tails >= 0 &&
