@@ -132,17 +132,22 @@ typedef struct pd_desc {
                             correction).  The result is the variant's approximation, so the
                             solve returns PD_OK without a convergence test.  0 = the full
                             method.  Single problems only (batch <= 1) */
-  /* Launch geometry; 0 selects the built-in choice (paradiag_autotune fills these). */
-  int32_t tune_pint_rows;    /* rows per thread of the shifted-solve kernel: 4, 8, or 16
-                                (16 with PD_MIXED only) */
-  int32_t tune_pint_teams;   /* teams (one tridiagonal block each) per CTA of that kernel:
+  /* Kernels and launch geometry; 0 selects the built-in choice (the Python autotuner fills
+   * these).  A nonzero tune_pint_rows, tune_pint_teams, tune_fft_cols or tune_fft_radix runs
+   * the general kernel it describes in place of the specialised built-in one. */
+  int32_t tune_pint_rows;    /* rows per thread of the general shifted-solve kernel: 4, 8, or 16
+                                (16 with PD_MIXED only).  The built-in choice keeps rows in
+                                registers (binary32) or gives each system a thread (FP64 plans
+                                of many systems) where it can */
+  int32_t tune_pint_teams;   /* teams (one tridiagonal block each) per CTA of the general kernel:
                                 a power of two with teams * threads-per-team <= 512
                                 (<= 256 with 16 rows per thread) */
   int32_t tune_krylov_ctas;  /* CTAs of the Krylov vector kernels: 1 = one 512-thread CTA
                                 (n_bar <= 8192), > 1 = cooperative launch of 512-thread CTAs
                                 (<= SM count) */
   int32_t tune_cap_ctas;     /* CTAs of the capacitance-term kernel, 1 .. 1024 */
-  int32_t tune_fft_cols;     /* columns per CTA of the time FFTs: 2, 4, 8 or 16 */
+  int32_t tune_fft_cols;     /* columns per CTA of the general time FFTs: 2, 4, 8 or 16 (0 also
+                                allows the register transforms of n_t = 32 .. 2048) */
   int32_t tune_no_pdl;       /* nonzero: launch kernels without programmatic dependent launch
                                 (by default a kernel may be scheduled while its predecessor
                                 drains; it waits for it before reading anything) */
@@ -181,8 +186,10 @@ typedef struct pd_desc {
   int32_t tune_fft_radix;    /* first stages of the time DFTs and the DST along y: 16 = one
                                 radix-16 stage in registers (n >= 16), then radix-4 passes in
                                 shared memory; 4 = radix-4 (and one radix-2) passes only;
-                                0 = built-in choice (16 for binary32 transforms of n >= 16, 4
-                                otherwise; the residual-on-load DFT always uses 4) */
+                                0 = built-in choice: the two-pass register transforms where they
+                                are built (n_t = 32 .. 2048, n_y = 63, 127, 255) and faster, else
+                                16 for binary32 transforms of n >= 16 and 4 otherwise (the general
+                                residual-on-load DFT always uses 4) */
   int32_t tune_persistent;   /* single problems: run each Algorithm-2 step after its shifted
                                 solves as one persistent cooperative launch (the eq. (12)
                                 terms and system, z, eq. (13) with the stopping decision, and

@@ -1,15 +1,18 @@
-"""Launch-geometry autotuner for one plan shape.
+"""Autotuner for one plan shape: kernels and launch geometry.
 
-Coordinate descent over the `tune_*` fields of pd_desc: rows per thread and teams per
-CTA of the shifted-solve kernel, columns per CTA and the first-stage radix (one radix-16
-stage in registers, or radix-4 passes only) of the time FFTs and the DST along y, CTAs of
-the capacitance-term kernel and of the Krylov vector kernels.  Each candidate plan solves
-the caller's right-hand side; its time is the median of CUDA-event timed solves with an
-L2 flush before each, and a candidate whose result differs from the default plan's by
+Coordinate descent over the `tune_*` fields of pd_desc.  0 keeps the built-in kernels; rows per thread
+and teams per CTA of the shifted solves run the general kernel (k_pint) in that geometry in place of the
+register and thread-per-system kernels, columns per CTA of the time FFTs and the first-stage radix of the
+FFTs and the DST along y (one radix-16 stage in registers, or radix-4 passes only) the general transforms
+in place of the two-pass register transforms.  The other fields set the CTAs of the capacitance-term
+kernel and of the Krylov vector kernels, their cluster and tails, and stored factors.
+Each candidate plan solves the caller's right-hand side; its time is the median of CUDA-event timed
+solves with an L2 flush before each, and a candidate whose result differs from the default plan's by
 more than the precision's tolerance is rejected.  Geometries the library refuses
 (PD_ERR_UNSUPPORTED / PD_ERR_INVALID_ARG) are skipped.  Results can be kept in a JSON
-cache file keyed by the plan shape and the GPU, so a shape is tuned once per machine.
-The tuner only chooses launch parameters; every solve runs in the library's kernels.
+cache file keyed by the plan shape, the GPU and the library's sources, so a shape is tuned once per
+machine and build.
+The tuner only chooses among the library's kernels and their launch parameters.
 """
 from __future__ import annotations
 
@@ -37,14 +40,17 @@ def _candidates(plan_kw, nf):
 
 
 def plan_key(plan) -> str:
-    """Cache key of a plan's shape: dimension, sizes, batch, precision and alpha, and the GPU
-    model (launch geometry depends on all of them)."""
+    """Cache key of a plan's shape: dimension, sizes, batch, precision and alpha, the GPU model and the
+    library's sources (the best choice depends on all of them; one measured on other kernels would keep
+    the shape off newer ones)."""
     import torch
+
+    from .build import source_digest
 
     d = plan.desc
     return json.dumps({"dim": plan.dim, "nx": plan.nx, "ny": plan.ny, "nt": plan.nt, "batch": plan.batch,
                        "precision": plan.precision, "alpha": float(d.alpha) or 1.0,
-                       "gpu": torch.cuda.get_device_name(plan.device)}, sort_keys=True)
+                       "gpu": torch.cuda.get_device_name(plan.device), "build": source_digest()}, sort_keys=True)
 
 
 def _cache_load(path):
@@ -70,7 +76,7 @@ def autotune(make_plan, G, reps=5, flush_bytes=256 << 20, log=None, cache=None):
 
     make_plan: callable taking tune=dict and returning a paper_2304_12597_gb300.Plan (used
     as a context manager).
-    cache: optional path of a JSON file.  A stored result for this plan's shape and GPU
+    cache: optional path of a JSON file.  A stored result for this plan's shape, GPU and build
     (plan_key) is returned without tuning; a new result is added to the file."""
     import torch
 

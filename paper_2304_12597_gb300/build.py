@@ -7,6 +7,7 @@ declared in include/paradiag.h.
 from __future__ import annotations
 
 import concurrent.futures as cf
+import hashlib
 import os
 import shutil
 import subprocess
@@ -32,6 +33,18 @@ def _flags(verbose_ptxas: bool):
     if verbose_ptxas:
         f += ["-Xptxas", "-v"]
     return f
+
+
+def source_digest() -> str:
+    """Identifies the kernels a tuned geometry was measured on: a digest of every source and header that
+    goes into the library."""
+    h = hashlib.sha256()
+    for path in [os.path.join(CSRC, f) for f in sorted(os.listdir(CSRC))] + [os.path.join(HERE, "..", "include", "paradiag.h")]:
+        if path.endswith((".cu", ".cuh", ".h")):
+            h.update(os.path.basename(path).encode() + b"\0")
+            with open(path, "rb") as f:
+                h.update(f.read())
+    return h.hexdigest()[:16]
 
 
 def _stale(target: str, deps) -> bool:
