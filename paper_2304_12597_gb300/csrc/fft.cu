@@ -520,7 +520,7 @@ __global__ void __launch_bounds__(256) k_fft_c2r(const cpx<T> *__restrict__ S, i
       ss = fmaf(vf, vf, ss);
     }
   }
-  c2r_finish<TX, 256>(ss, x0, ncols, colsum, norm_part, fin);
+  c2r_finish<TX, 256>((double)ss, x0, ncols, colsum, norm_part, fin);
 }
 
 // Orthonormal DST-I along y via a length N = 2(ny+1) complex FFT of the odd

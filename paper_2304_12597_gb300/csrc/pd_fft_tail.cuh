@@ -13,8 +13,10 @@ __device__ __forceinline__ void rhs_norm_finish(float ss, const RhsNorm &rn) {
   __shared__ double red[32];
   __shared__ int last;
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = blockDim.x >> 5;
-  ss = warp_sum(ss);  // binary32 within a warp (a reference scale; FP64 adds cost GB300's FP64 pipe)
-  if (l == 0) red[w] = (double)ss;
+  // binary32 within a warp (a reference scale; FP64 adds cost GB300's FP64 pipe), a quarter of it, so
+  // that a warp's up to 2048 squares overflow no earlier than 512 of their size would
+  ss = warp_sum(0.25f * ss);
+  if (l == 0) red[w] = 4.0 * (double)ss;
   __syncthreads();
   if (threadIdx.x == 0) {
     double t = 0.0;
@@ -44,13 +46,13 @@ __device__ __forceinline__ void rhs_norm_finish(float ss, const RhsNorm &rn) {
 // columns x0 .. x0 + TX - 1 going round the threads), per column and over the launch, and the
 // refinement decision in the last CTA (fin).  blockDim.x is a multiple of 32 and of TX, at most NT.
 template <int TX, int NT>
-__device__ __forceinline__ void c2r_finish(float ss, int64_t x0, int64_t ncols, double *colsum, double *norm_part,
+__device__ __forceinline__ void c2r_finish(double ss, int64_t x0, int64_t ncols, double *colsum, double *norm_part,
                                            const StepFinish &fin) {
   if (colsum) {
     // per-column sums of squares: blockDim.x is a multiple of TX, so every element a
     // thread wrote lies in column threadIdx.x % TX
     __shared__ double cred[NT];
-    cred[threadIdx.x] = (double)ss;
+    cred[threadIdx.x] = ss;
     __syncthreads();
     if ((int)threadIdx.x < TX) {
       double t = 0.0;
@@ -59,7 +61,7 @@ __device__ __forceinline__ void c2r_finish(float ss, int64_t x0, int64_t ncols, 
     }
   }
   if (norm_part) {
-    const double sd = warp_sum((double)ss);
+    const double sd = warp_sum(ss);
     __shared__ double red[32];
     const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
     __syncthreads();

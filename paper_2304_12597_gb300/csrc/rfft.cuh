@@ -182,7 +182,9 @@ __global__ void __launch_bounds__(rfft_threads<R1, R2, TX>(), rfft_ctas<T, R1, R
     ex = -sc.ex[b];
     dead = sc.zero[b] || col - (int64_t)b * sc.mnx >= sc.nxb[b];
   }
-  float ss = 0.0f;  // a few dozen squares per thread; the stop rule needs a few digits
+  // a few dozen squares per thread, in four sums of at most 16, so that binary32 overflows no earlier than
+  // with the 2 to 32 values per thread of fft.cu; the stop rule needs a few digits
+  float ss[4] = {0.0f, 0.0f, 0.0f, 0.0f};
   for (int r = it0; r < R2; r += NIT) {
     cpx<T> z[H];
     const cpx<T> *p = sm + r * H * TX;
@@ -216,12 +218,12 @@ __global__ void __launch_bounds__(rfft_threads<R1, R2, TX>(), rfft_ctas<T, R1, R
           vf = f64_to_f32_near(v);
         else
           vf = v;
-        ss = fmaf(vf, vf, ss);
+        ss[i % 4] = fmaf(vf, vf, ss[i % 4]);
       }
     }
   }
-  if (!live) ss = 0.0f;
-  c2r_finish<TX, NT>(ss, x0, ncols, colsum, norm_part, fin);
+  const float q = fmaf(0.25f, ss[0], 0.25f * ss[1]) + fmaf(0.25f, ss[2], 0.25f * ss[3]);
+  c2r_finish<TX, NT>(live ? f32_to_f64_bits(q, 2) : 0.0, x0, ncols, colsum, norm_part, fin);
 }
 
 // ---- dispatch -------------------------------------------------------------------------------
