@@ -111,7 +111,9 @@ typedef struct pd_desc {
                             first time step */
   double refine_tol;     /* refinement stops when the predicted remaining relative error,
                             (||delta_s|| / ||delta_{s-1}||) * ||delta_s|| / ||U||, is <= refine_tol
-                            (0 = 1e-14 for PD_FP64, 1e-11 for PD_MIXED) */
+                            (0 = 1e-14 for PD_FP64, 1e-11 for PD_MIXED); PD_MIXED also asks it of
+                            a tenth of sqrt(n_t) ||r_m|| / ||U||, the bound on what the sweep's own
+                            Algorithm 2 left (eq. 13) */
   double alpha;          /* alpha of Sec. 4 in (0, 1] (0 = 1): 1 runs Algorithm 1, alpha < 1
                             Algorithm 3 (alpha-circulant C_alpha, eq. 15: pi_k = alpha^{1/l}
                             omega^k, time rows scaled by D_alpha before the DFT and by

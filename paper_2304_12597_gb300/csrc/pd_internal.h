@@ -142,6 +142,14 @@ struct KrylovCtl {
   int maxit;
   int q;               // residual check every q steps (and at maxit or a breakdown)
 };
+// An inexact x_m leaves exactly -r_m in the first time step of eq. (2), so after a sweep whose
+// Algorithm 2 stopped with ||r_m|| the error is up to sqrt(n_t) ||r_m|| (what a contraction makes of
+// it over n_t steps), however fast the sweep before converged.  The ratio of the last updates does not
+// see it: in near-singular problems a sweep that met 1e-6 was followed by one that stalled, and the solve
+// stopped at a predicted 1e-14 with an error of 1.4e-8.  Measured error over this bound: 0.06 to 1 (heat
+// with open and almost insulated ends, alpha = 1).  A tenth of the bound, in units of ||delta_0||, is
+// asked to meet the tolerance.
+constexpr double kKrylovLeft = 0.1;
 struct RefineCtl {
   int fp64;
   double eps_first, eps_refine;  // Algorithm-2 tolerances of the first solve / sweeps
@@ -153,6 +161,10 @@ struct RefineCtl {
   int *msw;
   int *mconv;
   int member_solves;  // 0 = no per-problem limit (the plan's max_refine bounds the batch)
+  // PD_MIXED: kKrylovLeft sqrt(n_t), the weight of ||r_m||, else 0; batches read the problems' ||r_m||
+  // from their scalar blocks
+  double left;
+  const double *mscal;
 };
 // ---- time FFT / DST (fft.cu) ----------------------------------------------------
 // Forward DFT along time of real (n, ncols) rows -> half spectrum (n/2+1, ncols).

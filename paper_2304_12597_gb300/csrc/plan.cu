@@ -1253,6 +1253,8 @@ pd::RefineCtl refine_ctl(pd_plan *p) {
   r.msw = p->batch > 1 ? p->msw : nullptr;
   r.mconv = p->batch > 1 ? p->mconv : nullptr;
   r.member_solves = p->member_solves;
+  r.left = p->precision == PD_MIXED ? pd::kKrylovLeft * std::sqrt((double)p->nt) : 0.0;
+  r.mscal = p->batch > 1 ? p->mscal : nullptr;
   return r;
 }
 
