@@ -57,9 +57,9 @@ __global__ void __launch_bounds__(256) k_batch_sumsq(const double *__restrict__ 
 
 // ex[b] = -round(log2 ||slot b||_F): slot b is multiplied by 2^ex[b] before the solve
 // and its solution by 2^-ex[b] after it (0 for an all-zero or non-finite slot).
-// zero[b] = 1 for an all-zero slot: its solution is exactly zero, whatever rounding-level
-// values the paired real DFTs leave in its columns, and it takes no part in the
-// refinement decision.
+// zero[b] = 1 for an all-zero slot: its solution is stored as exact zeros, whatever rounding-level
+// values a transform that pairs columns (the DST, the general time DFTs) leaves in its columns, and
+// it takes no part in the refinement decision.
 __global__ void k_batch_exponents(int batch, int nc, const double *__restrict__ part, int *__restrict__ ex,
                                   int *__restrict__ zero, const double *G, const double **gslot) {
   grid_dep_wait();

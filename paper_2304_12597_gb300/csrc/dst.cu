@@ -20,7 +20,7 @@
 // The binary32 transforms move 200 to 333 MB at 255 x 255 x 256 (30 to 49 us of copy bandwidth); the
 // binary64 ones are bound by GB300's FP64 pipe.  With the residual on load, six FP64
 // operations per element bound both (33 us each at 255 x 255 x 256): binary32 261 -> 255 us,
-// binary64 1296 -> 773 us; a residual kernel of its own (231 us) beside the plain transform
+// binary64 1296 -> 864 us; a residual kernel of its own (231 us) beside the plain transform
 // (59 us) measured slower, since here the DST's passes of one CTA run beside the FP64 work of
 // the other.
 #include <algorithm>

@@ -780,11 +780,6 @@ __global__ void __launch_bounds__(kBlasSingle, 1) k_step_tail(StepArgs<T> a) {
 
 // ---- launchers -------------------------------------------------------------------
 
-// One CTA (plain launch) when the vector is short, else a cooperative launch through
-// cudaLaunchKernelEx (capturable into a CUDA graph).
-// Cluster variant: one CTA per SM (the dynamic shared memory request keeps a second
-// CTA off the SM), kBlasCluster threads each.
-//
 // Largest cluster size <= want (halving, down to 4: with 128 threads per CTA and at most
 // 16 register-held entries per thread, 4 CTAs cover the 8192 entries one CTA would
 // take) the device can co-schedule for the cluster variant of the vector kernels; 0 if
@@ -826,6 +821,9 @@ static int coop_elems(int n, int grid) {
                        : (E) == 4 ? (const void *)KERNEL<MODE, 4>                            \
                                   : (E) == 8 ? (const void *)KERNEL<MODE, 8> : (const void *)KERNEL<MODE, 16>)
 
+// One CTA (plain launch) when the vector is short, else a cooperative launch through
+// cudaLaunchKernelEx (capturable into a CUDA graph).  Cluster variant: one CTA per SM (the
+// dynamic shared memory request keeps a second CTA off the SM), kBlasCluster threads each.
 static void coop_launch(Ctx &c, const char *fam, double bytes, const void *fn_single, const void *fn_coop,
                         const void *fn_cluster, int grid, int cluster, void **args) {
   if (grid <= 1 && cluster > 1) {

@@ -30,10 +30,14 @@
 // (suits_excess in plan.cu; a graded symmetric operator with off-diagonals 600 times the diagonal
 // left the refinement short of convergence).
 //
-// What bounds it: instruction issue.  Against k_pint's two separators per chunk of 8 rows held
-// in shared memory this takes 16 rows per lane (half the PCR levels per row), keeps aa, cc, r
-// in registers, moves tau K as one 16-byte shared load per row, and prefetches the next
-// frequency's right-hand side with cp.async while this one is solved.
+// What bounds it: latency.  A lane walks a serial chain of 16 pivots, and at 168 registers an SM
+// holds 12 warps (14 % of its slots), which issue in 43 % of the cycles; wide teams (blocks of more
+// than 512 rows) also wait at a barrier per PCR level and for each frequency's loads.  104 thread
+// instructions per row at 255 rows a block, 156 at 4095.  Against k_pint's two separators per chunk
+// of 8 rows held in shared memory (230 instructions per row) this takes 16 rows per lane (half the PCR
+// levels per row), keeps aa, cc, r in registers, moves tau K as one 16-byte shared load per row, and,
+// up to teams of 128 lanes, prefetches the next frequency's right-hand side with cp.async while this
+// one is solved.
 // Measured per launch (one GB300, k_pint -> this kernel; b pass / h_k pass):
 //   2D 255 blocks of 255 rows, 129 frequencies     94 / 98 us   -> 45 / 41 us
 //   2D 127 blocks of 127 rows, 257 frequencies     67 / 71 us   -> 24 / 22 us

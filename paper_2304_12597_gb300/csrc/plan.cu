@@ -1067,12 +1067,12 @@ pd_status sync_read(pd_plan *p, bool last = false) {
   return ctx_status(p);
 }
 
-// The final loop by linearity applies to single problems of the full method whose zero
-// frequency runs in binary32 like the others (the FP64 lane keeps the final loop's solves).
 // Geometry of the loops of an Algorithm-1 solve: the FP64 zero-frequency lane is k_pint's, and so are
 // operators whose row sums say too little about their pivots.
 const pd::PintGeom &loop_geom(const pd_plan *p) { return p->excess && !p->lane ? p->cgeom : p->geom; }
 
+// The final loop by linearity applies to single problems of the full method whose zero
+// frequency runs in binary32 like the others (the FP64 lane keeps the final loop's solves).
 bool use_comb(const pd_plan *p) { return p->comb && !(p->precision == PD_MIXED && p->lane); }
 
 template <typename T>

@@ -1,7 +1,7 @@
 // Binary32, forward, of the 1D FP64 residual: the time DFT in registers (rfft.cuh) of
 // r_j = G_j + u_{j-1} - (I + tau K) u_j, formed while the tile is loaded.
 //
-// Bound by GB300's FP64 pipe (four operations per unknown: 4 us per million), with HBM well below it
+// Bound by GB300's FP64 pipe (four operations per unknown: 8 us per million), with HBM well below it
 // (20 bytes per unknown, 3 us per million).  The residual needs four loads per value, so it does not
 // suit pass 1, where a thread owns R1 rows and few threads run: all threads form it first, kRows
 // consecutive rows of one column at a time (u_{j-1} carries over), and leave it in shared memory as
