@@ -91,8 +91,10 @@ __device__ __forceinline__ void refine_decide(double *scal, int *flags, const Re
       const double rho = prev > 0.0 ? rel / prev : 0.0;
       const double pp = (s >= 3 && s < 16) ? scal[S_SWUPD + s - 2] : 0.0;
       const double rho_pred = pp > 0.0 ? fmax(rho, prev / pp) : rho;
-      const double left = r.left > 0.0 ? r.left * scal[S_RES] / sqrt(ref2) : 0.0;
-      if ((s >= 2 && fmax(rho_pred * rel, left) <= r.refine_tol && rel <= 1e-7) || rel <= 1e-15) {
+      const double left = r.left * scal[S_RES];  // (squares: no division or root on the decision's chain)
+      if ((s >= 2 && rho_pred * rel <= r.refine_tol && rel <= 1e-7 &&
+           (r.left == 0.0 || left * left <= r.refine_tol * r.refine_tol * ref2)) ||
+          rel <= 1e-15) {
         conv = stop = true;
       } else if (s > 1 && rho > 0.5) {  // no longer contracting: rounding floor reached
         conv = rel <= 1e-10;
@@ -151,9 +153,10 @@ __device__ __forceinline__ void refine_decide_members(double *scal, int *flags, 
       const double rho = prev[b] > 0.0 ? rel / prev[b] : 0.0;
       const bool floor_b = sb > 1 && rho > 0.5;  // no longer contracting: rounding floor
       // (||r_m|| is in the units of the sweep's residual, scaled by 2^mex[b])
-      const double left = r.left > 0.0 ? r.left * ldexp(r.mscal[(int64_t)b * kScalWords + S_RES], -mex[b]) / sqrt(rf) : 0.0;
+      const double left = r.left * r.mscal[(int64_t)b * kScalWords + S_RES];
+      const double tol = __hiloint2double((1023 + mex[b]) << 20, 0) * r.refine_tol;
       conv_b = sb > 0 &&
-               ((sb >= 2 && fmax(rho * rel, left) <= r.refine_tol && rel <= 1e-7) || rel <= 1e-15 || (floor_b && rel <= 1e-10));
+               ((sb >= 2 && rho * rel <= r.refine_tol && (r.left == 0.0 || left * left <= tol * tol * rf) && rel <= 1e-7) || rel <= 1e-15 || (floor_b && rel <= 1e-10));
       if (!conv_b) all_conv = false;
       if (!conv_b && floor_b) any_stall = true;  // stuck above the floor
       if (rel > 1e-10) all_floor = false;

@@ -31,9 +31,10 @@
 // left the refinement short of convergence).
 //
 // What bounds it: latency.  A lane walks a serial chain of 16 pivots, and at 168 registers an SM
-// holds 12 warps (14 % of its slots), which issue in 43 % of the cycles; wide teams (blocks of more
-// than 512 rows) also wait at a barrier per PCR level and for each frequency's loads.  104 thread
-// instructions per row at 255 rows a block, 156 at 4095.  Against k_pint's two separators per chunk
+// holds 12 warps (14 % of its slots), which issue in 49 % of the cycles (255 x 255 x 256); wide teams
+// (blocks of more than 512 rows; 16 warps, 42 % at 4095 x 2048) also wait at a barrier per PCR level
+// and, in one CTA of 256, for each frequency's loads.  105 thread instructions per row at 255 rows a
+// block, 156 at 4095.  Against k_pint's two separators per chunk
 // of 8 rows held in shared memory (230 instructions per row) this takes 16 rows per lane (half the PCR
 // levels per row), keeps aa, cc, r in registers, moves tau K as one 16-byte shared load per row, and,
 // up to teams of 128 lanes, prefetches the next frequency's right-hand side with cp.async while this
