@@ -947,8 +947,10 @@ size_t step_tail_smem(int maxit, int nf, int elem_bytes) {
   const size_t solve = (size_t)(2 * maxit * maxit + maxit) * sizeof(cpx<double>) + (size_t)(maxit + 1) * 8;
   const size_t wb = k5a_warp_bytes(maxit);
   const size_t terms = wb * std::max<size_t>(1, std::min<size_t>(kK5Warps, (150 * 1024) / wb));
+  // at m = 1 every warp of the CTA has a slice (few Krylov steps allowed: more than terms takes)
+  const size_t first = k5a_warp_bytes(1) * (kBlasSingle / 32);
   const size_t om = (size_t)nf * 2 * elem_bytes;
-  return (std::max(std::max(solve, terms), om) + 15) & ~(size_t)15;
+  return (std::max(std::max(solve, terms), std::max(first, om)) + 15) & ~(size_t)15;
 }
 
 // nv = 1: the vector phases in one CTA without grid barriers (E = 1: n_bar <= 512)
