@@ -92,9 +92,9 @@ __device__ __forceinline__ void refine_decide(double *scal, int *flags, const Re
       const double pp = (s >= 3 && s < 16) ? scal[S_SWUPD + s - 2] : 0.0;
       const double rho_pred = pp > 0.0 ? fmax(rho, prev / pp) : rho;
       const double left = r.left * scal[S_RES];  // (squares: no division or root on the decision's chain)
-      if ((s >= 2 && rho_pred * rel <= r.refine_tol && rel <= 1e-7 &&
-           (r.left == 0.0 || left * left <= r.refine_tol * r.refine_tol * ref2)) ||
-          rel <= 1e-15) {
+      const bool left_ok = r.left == 0.0 || left * left <= r.refine_tol * r.refine_tol * ref2;
+      // (an update whose squares underflow in binary32 reads as zero: ||r_m|| still says what is left)
+      if (left_ok && ((s >= 2 && rho_pred * rel <= r.refine_tol && rel <= 1e-7) || rel <= 1e-15)) {
         conv = stop = true;
       } else if (s > 1 && rho > 0.5) {  // no longer contracting: rounding floor reached
         conv = rel <= 1e-10;
@@ -156,7 +156,9 @@ __device__ __forceinline__ void refine_decide_members(double *scal, int *flags, 
       const double left = r.left * r.mscal[(int64_t)b * kScalWords + S_RES];
       const double tol = __hiloint2double((1023 + mex[b]) << 20, 0) * r.refine_tol;
       conv_b = sb > 0 &&
-               ((sb >= 2 && rho * rel <= r.refine_tol && (r.left == 0.0 || left * left <= tol * tol * rf) && rel <= 1e-7) || rel <= 1e-15 || (floor_b && rel <= 1e-10));
+               (((r.left == 0.0 || left * left <= tol * tol * rf) &&
+                 ((sb >= 2 && rho * rel <= r.refine_tol && rel <= 1e-7) || rel <= 1e-15)) ||
+                (floor_b && rel <= 1e-10));
       if (!conv_b) all_conv = false;
       if (!conv_b && floor_b) any_stall = true;  // stuck above the floor
       if (rel > 1e-10) all_floor = false;

@@ -41,6 +41,17 @@ def test_single_problems(pd, n, nt, T, seed):
     assert R.rel_err(U.cpu().numpy(), R.be_solve_refined(P)) <= 1e-10, st
 
 
+@pytest.mark.parametrize("scale", [2.0 ** -46, 2.0 ** -50])
+@pytest.mark.parametrize("n,nt,T,seed", [(200, 128, 1.3141721875863261, 162589093), (92, 8, 2.4997650143321515, 61807406),
+                                         (6, 4, 0.05245022822372974, 445)])
+def test_updates_below_the_range_of_binary32_squares(pd, n, nt, T, seed, scale):
+    """Right-hand sides so small that the squares of a sweep's update underflow in binary32."""
+    P = _insulated(n, nt, T, seed)
+    with pd.Plan.from_problem(P, precision="mixed") as plan:
+        U, st = plan.solve(torch.from_numpy(P.G * scale).cuda())
+    assert R.rel_err(U.cpu().numpy() / scale, R.be_solve_refined(P)) <= 1e-10, st
+
+
 @pytest.mark.parametrize("n,nt", [(3, 64), (117, 64), (200, 128), (79, 128)])
 @pytest.mark.parametrize("advance", [False, True])
 def test_batches(pd, n, nt, advance):
