@@ -1,5 +1,5 @@
 """The autotuner's cache key (no GPU): it names the library's sources, so that a result measured on other
-kernels is not taken for this build's."""
+kernels is not taken for the current ones."""
 import json
 import os
 import shutil
